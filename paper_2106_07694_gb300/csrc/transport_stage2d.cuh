@@ -13,7 +13,7 @@
 // a step (the stage-3 kernel also folds the floor deposit); c1 and c2 go through L2/HBM.
 #pragma once
 #include "common.cuh"
-#include "transport_sweep2d.cuh"  // weno5_face_value, face_flux_x
+#include "weno.cuh"
 
 namespace lw {
 
@@ -55,7 +55,7 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
   const int y0 = by * sp.H, y1 = min(ny, y0 + sp.H);
   const int X = (x0 + t) % nx;
   const bool out = x0 + t < nx;
-  const T inv_alpha = a.inv_alpha, vs_a = a.vs * a.inv_alpha, alpha = a.alpha, kappa = a.kappa;
+  const T inv_alpha = a.inv_alpha, vs_a = a.vs * a.inv_alpha, alpha = a.alpha, kd = a.kappa * a.inv_alpha;
   const T* __restrict__ cin = sp.cin;
   const T* __restrict__ ux = a.u;
   const T* __restrict__ uy = a.u + a.n;
@@ -140,12 +140,12 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
     if (!prime) {
       if constexpr (SCHEME == 0) {
         S.fx[t] = face_flux_x(S.xp[t], S.xp[t + 1], S.xp[t + 2], S.xp[t + 3], S.xp[t + 4], S.xm[t + 5],
-                              S.xm[t + 4], S.xm[t + 3], S.xm[t + 2], S.xm[t + 1], alpha, kappa, S.c[t + kS2h - 1],
+                              S.xm[t + 4], S.xm[t + 3], S.xm[t + 2], S.xm[t + 1], kd, S.c[t + kS2h - 1],
                               S.c[t + kS2h]);
         if (t == 0) {
           const int e = kS2T;
           S.fx[e] = face_flux_x(S.xp[e], S.xp[e + 1], S.xp[e + 2], S.xp[e + 3], S.xp[e + 4], S.xm[e + 5],
-                                S.xm[e + 4], S.xm[e + 3], S.xm[e + 2], S.xm[e + 1], alpha, kappa, S.c[e + kS2h - 1],
+                                S.xm[e + 4], S.xm[e + 3], S.xm[e + 2], S.xm[e + 1], kd, S.c[e + kS2h - 1],
                                 S.c[e + kS2h]);
         }
       } else {
@@ -156,7 +156,7 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
             p[q] = S.xp[j + q];
             m[q] = S.xm[j + q];
           }
-          return face_flux_scheme<SCHEME>(p, m, alpha, kappa, S.c[j + kS2h - 1], S.c[j + kS2h]);
+          return face_flux_scheme<SCHEME>(p, m, kd, S.c[j + kS2h - 1], S.c[j + kS2h]);
         };
         S.fx[t] = xface(t);
         if (t == 0) S.fx[kS2T] = xface(kS2T);
@@ -170,7 +170,7 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
       const T* M = &S.ym[rb][t];
       if constexpr (SCHEME == 0) {
         fup = face_flux_x(P[0], P[kS2T], P[2 * kS2T], P[3 * kS2T], P[4 * kS2T], M[5 * kS2T], M[4 * kS2T],
-                          M[3 * kS2T], M[2 * kS2T], M[kS2T], alpha, kappa, chere, cnext);
+                          M[3 * kS2T], M[2 * kS2T], M[kS2T], kd, chere, cnext);
       } else {
         T p[6], m[6];
 #pragma unroll
@@ -178,7 +178,7 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
           p[q] = P[q * kS2T];
           m[q] = M[q * kS2T];
         }
-        fup = face_flux_scheme<SCHEME>(p, m, alpha, kappa, chere, cnext);
+        fup = face_flux_scheme<SCHEME>(p, m, kd, chere, cnext);
       }
     }
     __syncthreads();
@@ -186,18 +186,10 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
     // ---- divergence and the Shu-Osher combination of this stage
     if (!prime) {
       const T vs_floor = SUGAR && k == 0 ? a.vs * fma_t(-a.ks, __ldg(a.S + X), T(1)) : a.vs;
-      const T fdn = k == 0 ? -vs_floor * chere : carry;
-      const T L = S.fx[t] - S.fx[t + 1] + fdn - fup;
+      const T Lk = S.fx[t] - S.fx[t + 1] + carry - fup;  // carry is 0 below the floor row
+      const T cb = k == 0 ? fma_t(-vs_floor, chere, chere) : chere;  // less the floor outflow
       if (out) {
-        T v;
-        if (STAGE == 1) {
-          v = chere + L;
-        } else if (STAGE == 2) {
-          v = fma_t(T(0.75), cn_here, T(0.25) * (chere + L));
-        } else {
-          const T s = chere + L;
-          v = fma_t(T(1) / T(3), cn_here - s, s);
-        }
+        const T v = rk_combine<STAGE>(cb, Lk, alpha, cn_here);
         sp.cout[(unsigned)k * (unsigned)nx + X] = v;
         if (STAGE == 3) {
           report_status(a.status, !isfinite(v));

@@ -18,11 +18,11 @@
 //    ahead; the lower y face is carried from the previous row;
 //  - stages 2 and 3 also combine with c^n at the node, copied two rows ahead by cp.async
 //    into a three-row ring in shared memory (no registers held while it is in flight).
-// Every face is computed once, with the arithmetic of weno5_face_value/face_flux_x, so
+// Every face is computed once, with the arithmetic of face_flux_x, so
 // the faces and the updated c are bitwise those of the one-column kernel.
 #pragma once
 #include "common.cuh"
-#include "transport_sweep2d.cuh"  // weno5_q, weno5_face_value, face_flux_x
+#include "weno.cuh"
 #include "transport_stage2d.cuh"  // Stage2dParams
 
 namespace lw {
@@ -67,7 +67,7 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
   const int xl = x0 + kWq * t;  // first column of this thread (past a ragged strip end: wrapped)
   const bool out = xl < nx;
   const unsigned X = (unsigned)(xl % nx);
-  const float ia = a.inv_alpha, vs_a = a.vs * a.inv_alpha, alpha = a.alpha, kappa = a.kappa;
+  const float ia = a.inv_alpha, vs_a = a.vs * a.inv_alpha, alpha = a.alpha, kd = a.kappa * a.inv_alpha;
   const float* __restrict__ cin = sp.cin;
   const float* __restrict__ ux = a.u;
   const float* __restrict__ uy = a.u + a.n;
@@ -142,7 +142,7 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
         C[o] = LD::s(cin + row + col);
         lf_split(C[o], LD::s(ux + row + col) * ia, P[o], M[o]);
       }
-      e = face_flux_x(P[0], P[1], P[2], P[3], P[4], M[5], M[4], M[3], M[2], M[1], alpha, kappa, C[2], C[3]);
+      e = face_flux_x(P[0], P[1], P[2], P[3], P[4], M[5], M[4], M[3], M[2], M[1], kd, C[2], C[3]);
     }
     S.edge[r] = e;
   }
@@ -202,11 +202,9 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
       }
 #pragma unroll
       for (int f = 0; f < 4; ++f) {  // face between columns x - 1 + f and x + f
-        const float hp = fmaf(weno5_q(D[f], D[f + 1], D[f + 2], D[f + 3], SD[f], SD[f + 1], SD[f + 2]),
-                              1.f / 6.f, P[f + 2]);
-        const float hm = fmaf(weno5_q(-E[f + 3], -E[f + 2], -E[f + 1], -E[f], SE[f + 2], SE[f + 1], SE[f]),
-                              1.f / 6.f, M[f + 2]);
-        fxq[f] = fmaf(alpha, hp + hm, kappa * (C[f] - C[f + 1]));
+        const Recon<float> hp = weno5_recon(D[f], D[f + 1], D[f + 2], D[f + 3], SD[f], SD[f + 1], SD[f + 2]);
+        const Recon<float> hm = weno5_recon(-E[f + 3], -E[f + 2], -E[f + 1], -E[f], SE[f + 2], SE[f + 1], SE[f]);
+        fxq[f] = fmaf(kd, C[f] - C[f + 1], recon_sum(hp, P[f + 2], hm, M[f + 2]));
       }
       S.fx[b][t] = fxq[0];
       if (t == kWT - 1) S.fx[b][kWT] = S.edge[k - y0];
@@ -219,10 +217,10 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
                    P3 = ring_at(S.yp, ring[3]), P4 = ring_at(S.yp, ring[4]);
       const float4 M1 = ring_at(S.ym, ring[1]), M2 = ring_at(S.ym, ring[2]), M3 = ring_at(S.ym, ring[3]),
                    M4 = ring_at(S.ym, ring[4]), M5 = ring_at(S.ym, ring[5]);
-      fup[0] = face_flux_x(P0.x, P1.x, P2.x, P3.x, P4.x, M5.x, M4.x, M3.x, M2.x, M1.x, alpha, kappa, cq.x, cnext.x);
-      fup[1] = face_flux_x(P0.y, P1.y, P2.y, P3.y, P4.y, M5.y, M4.y, M3.y, M2.y, M1.y, alpha, kappa, cq.y, cnext.y);
-      fup[2] = face_flux_x(P0.z, P1.z, P2.z, P3.z, P4.z, M5.z, M4.z, M3.z, M2.z, M1.z, alpha, kappa, cq.z, cnext.z);
-      fup[3] = face_flux_x(P0.w, P1.w, P2.w, P3.w, P4.w, M5.w, M4.w, M3.w, M2.w, M1.w, alpha, kappa, cq.w, cnext.w);
+      fup[0] = face_flux_x(P0.x, P1.x, P2.x, P3.x, P4.x, M5.x, M4.x, M3.x, M2.x, M1.x, kd, cq.x, cnext.x);
+      fup[1] = face_flux_x(P0.y, P1.y, P2.y, P3.y, P4.y, M5.y, M4.y, M3.y, M2.y, M1.y, kd, cq.y, cnext.y);
+      fup[2] = face_flux_x(P0.z, P1.z, P2.z, P3.z, P4.z, M5.z, M4.z, M3.z, M2.z, M1.z, kd, cq.z, cnext.z);
+      fup[3] = face_flux_x(P0.w, P1.w, P2.w, P3.w, P4.w, M5.w, M4.w, M3.w, M2.w, M1.w, kd, cq.w, cnext.w);
     }
     // ---- ring: row k + 4 replaces row k - 2; fetch row k + 5
     put_r(ring[0]);
@@ -246,20 +244,13 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
       const float ch[4] = {cq.x, cq.y, cq.z, cq.w};
       const float cnv[4] = {cn.x, cn.y, cn.z, cn.w};
       const float cy[4] = {carry.x, carry.y, carry.z, carry.w};
-      float v[4];
+      float v[4], cb[4] = {ch[0], ch[1], ch[2], ch[3]};
+      if (k == 0) {  // the floor row's settling outflow (its lower face, carry, is 0)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float fdn = k == 0 ? -a.vs * ch[j] : cy[j];
-        const float L = fxq[j] - fr[j] + fdn - fup[j];
-        if (STAGE == 1) {
-          v[j] = ch[j] + L;
-        } else if (STAGE == 2) {
-          v[j] = fmaf(0.75f, cnv[j], 0.25f * (ch[j] + L));
-        } else {
-          const float s = ch[j] + L;
-          v[j] = fmaf(1.f / 3.f, cnv[j] - s, s);
-        }
+        for (int j = 0; j < 4; ++j) cb[j] = fmaf(-a.vs, ch[j], ch[j]);
       }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = rk_combine<STAGE>(cb[j], fxq[j] - fr[j] + cy[j] - fup[j], alpha, cnv[j]);
       if (out) {
         *reinterpret_cast<float4*>(sp.cout + (unsigned)k * (unsigned)nx + X) = make_float4(v[0], v[1], v[2], v[3]);
         if (STAGE == 3) {

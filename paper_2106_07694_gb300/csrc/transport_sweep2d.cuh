@@ -14,10 +14,8 @@
 // halo overlap.
 //
 // Arithmetic.  Scalar FP32 (packed f32x2 instructions issue to the FP64 pipe on
-// this part, which is far narrower).  The WENO5-JS reconstruction is written on
-// first differences with a single division per face half.  Split fluxes are kept
-// divided by alpha (epsilon = 1e-6 alpha^2 on the unscaled flux, as in the generic
-// kernel).
+// this part, which is far narrower); the reconstruction is that of weno.cuh on split fluxes
+// kept divided by alpha.
 //
 // Walls.  Ghost rows -2, -1 and ny, ny+1 hold the even reflection of c and the odd
 // reflection of the fluid velocity (Vs unchanged); the floor face carries -Vs c_0,
@@ -29,130 +27,11 @@
 #pragma once
 #include "common.cuh"
 #include "reduce_kernels.cuh"
+#include "weno.cuh"
 
 #include <type_traits>
 
 namespace lw {
-
-// ---------------------------------------------------------------- WENO5-JS, scalar FP32
-// Written on the first differences d1..d4 of the five upwind-side values a..e, which
-// the smoothness indicators and the three candidates share:
-//   beta_0 = 13/12 (d2-d1)^2 + 1/4 (3 d2 - d1)^2,  beta_1 = 13/12 (d3-d2)^2 + 1/4 (d2+d3)^2,
-//   beta_2 = 13/12 (d4-d3)^2 + 1/4 (d4 - 3 d3)^2;
-//   6 (q_k - c) = 5 d2 - 2 d1,  d2 + 2 d3,  4 d3 - d4;
-// and one division.  The weights are proportional to d_k prod_{j != k} A_j with
-// A_k = (eps + beta_k)^2, and only their ratios matter, so beta_k and eps are both scaled
-// by 12/13 (beta_k' = s_k^2 + 3/13 t_k^2) and the linear weights (1, 6, 3)/10 by 10:
-//   q-weights  A1 A2,  6 A0 A2,  3 A0 A1;
-//   numerator  A1 (A2 r0 + 3 A0 r2) + 6 A0 A2 r1,  denominator  A1 (A2 + 3 A0) + 6 A0 A2.
-// Returns the face value c + sum_k w_k (q_k - c).
-//
-// weno5_q takes the differences d1..d4 and the second differences s_k = d_{k+2} - d_{k+1}
-// and returns 6 sum_k w_k (q_k - c) = num / den, so that kernels which reconstruct several
-// adjacent faces can share the differences between them.  Rounding is sign-symmetric, so
-// b - a = -(a - b) bit for bit: a mirrored (h-) reconstruction may pass the negated
-// differences of the stored order and gets the same bits as weno5_face_value.
-__device__ __forceinline__ float weno5_q(float d1, float d2, float d3, float d4, float s0, float s1, float s2) {
-  const float t0 = fmaf(3.f, d2, -d1), t1 = d2 + d3, t2 = fmaf(-3.f, d3, d4);
-  const float q = 3.f / 13.f, eps = 1e-6f * (12.f / 13.f);
-  float A0 = fmaf(s0, s0, fmaf(q * t0, t0, eps));
-  float A1 = fmaf(s1, s1, fmaf(q * t1, t1, eps));
-  float A2 = fmaf(s2, s2, fmaf(q * t2, t2, eps));
-  A0 *= A0;
-  A1 *= A1;
-  A2 *= A2;
-  const float r0 = fmaf(5.f, d2, -2.f * d1), r1 = fmaf(2.f, d3, d2), r2 = fmaf(4.f, d3, -d4);
-  const float A02x6 = 6.f * (A0 * A2);
-  const float num = fmaf(A1, fmaf(3.f * A0, r2, A2 * r0), A02x6 * r1);
-  const float den = fmaf(A1, fmaf(3.f, A0, A2), A02x6);
-  return __fdividef(num, den);
-}
-
-__device__ __forceinline__ float weno5_face_value(float a, float b, float c, float d, float e) {
-  const float d1 = b - a, d2 = c - b, d3 = d - c, d4 = e - d;
-  return fmaf(weno5_q(d1, d2, d3, d4, d2 - d1, d3 - d2, d4 - d3), 1.f / 6.f, c);
-}
-
-// The paper's third-order WENO face value (Supplement Eqs. S10, S11, S14-S16) on the
-// upwind-side values a, b, c = h_{i-1}, h_i, h_{i+1}: candidates (b + c)/2 and (3b - a)/2,
-// indicators (c - b)^2 and (b - a)^2, linear weights 2/3 and 1/3; one division.
-__device__ __forceinline__ float weno3_face_value(float a, float b, float c) {
-  const float eps = 1e-6f;
-  float a1 = fmaf(c - b, c - b, eps), a2 = fmaf(b - a, b - a, eps);
-  a1 *= a1;
-  a2 *= a2;
-  const float p1 = 2.f * a2;  // (2/3)/a1 : (1/3)/a2 over the common factor 1/(3 a1 a2)
-  return __fdividef(fmaf(p1, b + c, a1 * fmaf(3.f, b, -a)), 2.f * (p1 + a1));
-}
-
-// FP64 forms of the same face values (the validation build): the same algebra with fma
-// and an IEEE division.
-__device__ __forceinline__ double weno5_q(double d1, double d2, double d3, double d4, double s0, double s1,
-                                          double s2) {
-  const double t0 = fma(3.0, d2, -d1), t1 = d2 + d3, t2 = fma(-3.0, d3, d4);
-  const double q = 3.0 / 13.0, eps = 1e-6 * (12.0 / 13.0);
-  double A0 = fma(s0, s0, fma(q * t0, t0, eps));
-  double A1 = fma(s1, s1, fma(q * t1, t1, eps));
-  double A2 = fma(s2, s2, fma(q * t2, t2, eps));
-  A0 *= A0;
-  A1 *= A1;
-  A2 *= A2;
-  const double r0 = fma(5.0, d2, -2.0 * d1), r1 = fma(2.0, d3, d2), r2 = fma(4.0, d3, -d4);
-  const double A02x6 = 6.0 * (A0 * A2);
-  const double num = fma(A1, fma(3.0 * A0, r2, A2 * r0), A02x6 * r1);
-  const double den = fma(A1, fma(3.0, A0, A2), A02x6);
-  return num / den;
-}
-
-__device__ __forceinline__ double weno5_face_value(double a, double b, double c, double d, double e) {
-  const double d1 = b - a, d2 = c - b, d3 = d - c, d4 = e - d;
-  return fma(weno5_q(d1, d2, d3, d4, d2 - d1, d3 - d2, d4 - d3), 1.0 / 6.0, c);
-}
-
-__device__ __forceinline__ double weno3_face_value(double a, double b, double c) {
-  const double eps = 1e-6;
-  double a1 = fma(c - b, c - b, eps), a2 = fma(b - a, b - a, eps);
-  a1 *= a1;
-  a2 *= a2;
-  const double p1 = 2.0 * a2;
-  return fma(p1, b + c, a1 * fma(3.0, b, -a)) / (2.0 * (p1 + a1));
-}
-
-// Face flux of a transport-scheme variant (SCHEME = kSchemeWeno3 | kSchemeSignSplit bits;
-// 0 is the Lax-Friedrichs WENO5 of face_flux_x) from the staged pairs of the six points
-// i-2 .. i+3 around the face i+1/2 (p[k], m[k] = point i-2+k).  Lax-Friedrichs schemes
-// stage p = h+/alpha, m = h-/alpha; the sign split stages p = w c/alpha, m = w/alpha and
-// reconstructs w c from the side the face velocity (w_i + w_{i+1})/2 comes from (ties
-// to the left).  T = float or double.
-template <int SCHEME, typename T>
-__device__ __forceinline__ T face_flux_scheme(const T (&p)[6], const T (&m)[6], T alpha, T kappa, T cl, T cr) {
-  constexpr bool W3 = (SCHEME & kSchemeWeno3) != 0, SIGN = (SCHEME & kSchemeSignSplit) != 0;
-  T h;
-  if (SIGN) {
-    const bool left = m[2] + m[3] >= T(0);
-    if (W3) {
-      h = weno3_face_value(left ? p[1] : p[4], left ? p[2] : p[3], left ? p[3] : p[2]);
-    } else {
-      h = weno5_face_value(left ? p[0] : p[5], left ? p[1] : p[4], left ? p[2] : p[3], left ? p[3] : p[2],
-                           left ? p[4] : p[1]);
-    }
-  } else if (W3) {
-    h = weno3_face_value(p[1], p[2], p[3]) + weno3_face_value(m[4], m[3], m[2]);
-  } else {
-    h = weno5_face_value(p[0], p[1], p[2], p[3], p[4]) + weno5_face_value(m[5], m[4], m[3], m[2], m[1]);
-  }
-  return fma_t(alpha, h, kappa * (cl - cr));
-}
-
-// Total face flux (unscaled): alpha (h+ + h-) + kappa (cl - cr), with h+ from the
-// left-biased values p0..p4 and h- from the right-biased values m0..m4 (already mirrored).
-template <typename T>
-__device__ __forceinline__ T face_flux_x(T p0, T p1, T p2, T p3, T p4, T m0, T m1, T m2, T m3, T m4, T alpha, T kappa,
-                                         T cl, T cr) {
-  const T hp = weno5_face_value(p0, p1, p2, p3, p4);
-  const T hm = weno5_face_value(m0, m1, m2, m3, m4);
-  return fma_t(alpha, hp + hm, kappa * (cl - cr));
-}
 
 // ---------------------------------------------------------------- geometry / smem
 
@@ -202,13 +81,13 @@ __device__ __forceinline__ void put_splits(SweepSmem& S, int stage, int row, int
   S.ym[stage][ry][t] = fmaf(wy, h, -h);
 }
 
-// Left x-face flux of column t at `row` for a stage (reads its x-split ring).
+// Left x-face flux of column t at `row` for a stage (reads its x-split ring); kd = kappa / alpha.
 __device__ __forceinline__ float xface(const SweepSmem& S, int stage, const float* crow, int row, int t,
-                                       float alpha, float kappa) {
+                                       float alpha, float kd) {
   const float* P = S.xp[stage][row & (kRx - 1)] + kSwPad + t;
   const float* M = S.xm[stage][row & (kRx - 1)] + kSwPad + t;
-  return face_flux_x(P[-3], P[-2], P[-1], P[0], P[1], M[2], M[1], M[0], M[-1], M[-2], alpha, kappa,
-                     crow[kSwPad + t - 1], crow[kSwPad + t]);
+  return alpha * face_flux_x(P[-3], P[-2], P[-1], P[0], P[1], M[2], M[1], M[0], M[-1], M[-2], kd, crow[kSwPad + t - 1],
+                             crow[kSwPad + t]);
 }
 
 // Upper y-face flux (row + 1/2) of column t for a stage (reads its y-split ring).
@@ -231,7 +110,7 @@ __device__ __forceinline__ void y_split(const SweepSmem& S, int stage, int rr, i
 
 // yo[k] = slot of row (row - 2 + k) in the stage's y ring, k = 0..5.
 __device__ __forceinline__ float yface(const SweepSmem& S, int stage, int row, int t, int ny, float sigma,
-                                       const int (&yo)[6], float alpha, float kappa, float c_here,
+                                       const int (&yo)[6], float alpha, float kd, float c_here,
                                        float c_above) {
   const float* P = &S.yp[stage][0][t];
   const float* M = &S.ym[stage][0][t];
@@ -243,12 +122,11 @@ __device__ __forceinline__ float yface(const SweepSmem& S, int stage, int row, i
       y_split(S, stage, row - 2 + k, t, ny, sigma, p[k], dummy);
       y_split(S, stage, row + 3 - k, t, ny, sigma, dummy, m[k]);
     }
-    return face_flux_x(p[0], p[1], p[2], p[3], p[4], m[0], m[1], m[2], m[3], m[4], alpha, kappa, c_here,
-                       c_above);
+    return alpha * face_flux_x(p[0], p[1], p[2], p[3], p[4], m[0], m[1], m[2], m[3], m[4], kd, c_here, c_above);
   }
   const int R = kSwThreads;
-  return face_flux_x(P[yo[0] * R], P[yo[1] * R], P[yo[2] * R], P[yo[3] * R], P[yo[4] * R], M[yo[5] * R],
-                     M[yo[4] * R], M[yo[3] * R], M[yo[2] * R], M[yo[1] * R], alpha, kappa, c_here, c_above);
+  return alpha * face_flux_x(P[yo[0] * R], P[yo[1] * R], P[yo[2] * R], P[yo[3] * R], P[yo[4] * R], M[yo[5] * R],
+                             M[yo[4] * R], M[yo[3] * R], M[yo[2] * R], M[yo[1] * R], kd, c_here, c_above);
 }
 
 __global__ void __launch_bounds__(kSwThreads, 2) rk3_sweep2d_kernel(Args<float> a, SweepParams sp) {
@@ -262,7 +140,7 @@ __global__ void __launch_bounds__(kSwThreads, 2) rk3_sweep2d_kernel(Args<float> 
   const bool out_col = t >= kSwHalo && t < kSwHalo + sp.W && (x0 + t - kSwHalo) < nx;
   const int y0 = blockIdx.y * sp.H;
   const int y1 = min(ny, y0 + sp.H);
-  const float kappa = a.kappa, alpha = sp.alpha, vs = a.vs;
+  const float alpha = sp.alpha, vs = a.vs, kd = a.kappa * a.inv_alpha;
   const float inv_alpha = a.inv_alpha, vs_a = a.vs * a.inv_alpha, sigma = 0.5f * sp.ghost_shift;
   const float* __restrict__ cin = a.c + X;
   const float* __restrict__ ux = a.u + X;
@@ -319,9 +197,9 @@ __global__ void __launch_bounds__(kSwThreads, 2) rk3_sweep2d_kernel(Args<float> 
     const int c0s2 = r2 & (kRc0 - 1), c0s3 = r3 & (kRc0 - 1);
 
     // ---- phase A: x faces of the three stages (data from earlier rows) and the new input row
-    if (act1) S.fx[par][0][kSwPad + t] = xface(S, 0, S.c0[c0s1], r1, t, alpha, kappa);
-    if (act2) S.fx[par][1][kSwPad + t] = xface(S, 1, S.c1[r2 & (kRc - 1)], r2, t, alpha, kappa);
-    if (act3) S.fx[par][2][kSwPad + t] = xface(S, 2, S.c2[r3 & (kRc - 1)], r3, t, alpha, kappa);
+    if (act1) S.fx[par][0][kSwPad + t] = xface(S, 0, S.c0[c0s1], r1, t, alpha, kd);
+    if (act2) S.fx[par][1][kSwPad + t] = xface(S, 1, S.c1[r2 & (kRc - 1)], r2, t, alpha, kd);
+    if (act3) S.fx[par][2][kSwPad + t] = xface(S, 2, S.c2[r3 & (kRc - 1)], r3, t, alpha, kd);
     if (r0 <= r_load_end) {
       const float c = qc[par], vx = qx[par], vy = qy[par];
       fetch(r0 + 2, qc[par], qx[par], qy[par]);
@@ -342,7 +220,7 @@ __global__ void __launch_bounds__(kSwThreads, 2) rk3_sweep2d_kernel(Args<float> 
     if (act1 || prime1) {
       const float chere = S.c0[c0s1][kSwPad + t];
       const float fup =
-          (r1 == ny - 1) ? 0.f : yface(S, 0, r1, t, ny, sigma, yo13, alpha, kappa, chere, S.c0[c0s1u][kSwPad + t]);
+          (r1 == ny - 1) ? 0.f : yface(S, 0, r1, t, ny, sigma, yo13, alpha, kd, chere, S.c0[c0s1u][kSwPad + t]);
       if (act1) {
         const float fdn = (r1 == 0) ? -vs * chere : carry[0];
         const float L = S.fx[par][0][kSwPad + t] - S.fx[par][0][kSwPad + t + 1] + fdn - fup;
@@ -366,7 +244,7 @@ __global__ void __launch_bounds__(kSwThreads, 2) rk3_sweep2d_kernel(Args<float> 
     if (act2 || prime2) {
       const float chere = S.c1[r2 & (kRc - 1)][kSwPad + t];
       const float fup = (r2 == ny - 1) ? 0.f
-                                       : yface(S, 1, r2, t, ny, sigma, yo2, alpha, kappa, chere,
+                                       : yface(S, 1, r2, t, ny, sigma, yo2, alpha, kd, chere,
                                                S.c1[(r2 + 1) & (kRc - 1)][kSwPad + t]);
       if (act2) {
         const float fdn = (r2 == 0) ? -vs * chere : carry[1];
@@ -388,7 +266,7 @@ __global__ void __launch_bounds__(kSwThreads, 2) rk3_sweep2d_kernel(Args<float> 
     if (act3 || prime3) {
       const float chere = S.c2[r3 & (kRc - 1)][kSwPad + t];
       const float fup = (r3 == ny - 1) ? 0.f
-                                       : yface(S, 2, r3, t, ny, sigma, yo13, alpha, kappa, chere,
+                                       : yface(S, 2, r3, t, ny, sigma, yo13, alpha, kd, chere,
                                                S.c2[(r3 + 1) & (kRc - 1)][kSwPad + t]);
       if (act3) {
         const float fdn = (r3 == 0) ? -vs * chere : carry[2];

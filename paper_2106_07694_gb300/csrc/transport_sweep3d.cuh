@@ -15,7 +15,7 @@
 // and the fluid velocity (odd, Vs unchanged); the floor face carries -Vs c(0), the lid 0.
 #pragma once
 #include "common.cuh"
-#include "transport_sweep2d.cuh"  // weno5_face_value, face_flux_x
+#include "weno.cuh"
 
 namespace lw {
 
@@ -59,7 +59,7 @@ __device__ __forceinline__ void rk_sweep3d_body(const Args<float>& a, const Swee
   const int X = (x0 + tx) % nx, Y = (y0 + ty) % ny;
   const bool out = (x0 + tx) < nx && (y0 + ty) < ny;
   const unsigned plane = (unsigned)nx * (unsigned)ny, n = (unsigned)a.n;
-  const float inv_alpha = a.inv_alpha, vs_a = a.vs * a.inv_alpha, alpha = a.alpha, kappa = a.kappa;
+  const float inv_alpha = a.inv_alpha, vs_a = a.vs * a.inv_alpha, alpha = a.alpha, kd = a.kappa * a.inv_alpha;
   const float* __restrict__ cin = sp.cin;
   const float* __restrict__ ux = a.u;
   const float* __restrict__ uy = a.u + n;
@@ -169,22 +169,21 @@ __device__ __forceinline__ void rk_sweep3d_body(const Args<float>& a, const Swee
       if (!prime) {
         const float* P = &S.xp[ty][tx];
         const float* M = &S.xm[ty][tx];
-        S.fx[ty][tx] = face_flux_x(P[0], P[1], P[2], P[3], P[4], M[5], M[4], M[3], M[2], M[1], alpha, kappa,
+        S.fx[ty][tx] = face_flux_x(P[0], P[1], P[2], P[3], P[4], M[5], M[4], M[3], M[2], M[1], kd,
                                    S.c[ty + kT3h][tx + kT3h - 1], S.c[ty + kT3h][tx + kT3h]);
         S.fy[ty][tx] = face_flux_x(S.yp[ty][tx], S.yp[ty + 1][tx], S.yp[ty + 2][tx], S.yp[ty + 3][tx],
                                    S.yp[ty + 4][tx], S.ym[ty + 5][tx], S.ym[ty + 4][tx], S.ym[ty + 3][tx],
-                                   S.ym[ty + 2][tx], S.ym[ty + 1][tx], alpha, kappa, S.c[ty + kT3h - 1][tx + kT3h],
+                                   S.ym[ty + 2][tx], S.ym[ty + 1][tx], kd, S.c[ty + kT3h - 1][tx + kT3h],
                                    S.c[ty + kT3h][tx + kT3h]);
         if (ty == 0 && tx < kT3y) {  // right edge x faces (column 32) of the tile rows
           const float* Pe = &S.xp[tx][kT3x];
           const float* Me = &S.xm[tx][kT3x];
-          S.fx[tx][kT3x] = face_flux_x(Pe[0], Pe[1], Pe[2], Pe[3], Pe[4], Me[5], Me[4], Me[3], Me[2], Me[1], alpha,
-                                       kappa, S.c[tx + kT3h][kT3x + kT3h - 1], S.c[tx + kT3h][kT3x + kT3h]);
+          S.fx[tx][kT3x] = face_flux_x(Pe[0], Pe[1], Pe[2], Pe[3], Pe[4], Me[5], Me[4], Me[3], Me[2], Me[1], kd, S.c[tx + kT3h][kT3x + kT3h - 1], S.c[tx + kT3h][kT3x + kT3h]);
         }
         if (ty == 1) {  // upper edge y faces (row 8) of the tile columns
           S.fy[kT3y][tx] = face_flux_x(S.yp[kT3y][tx], S.yp[kT3y + 1][tx], S.yp[kT3y + 2][tx], S.yp[kT3y + 3][tx],
                                        S.yp[kT3y + 4][tx], S.ym[kT3y + 5][tx], S.ym[kT3y + 4][tx],
-                                       S.ym[kT3y + 3][tx], S.ym[kT3y + 2][tx], S.ym[kT3y + 1][tx], alpha, kappa,
+                                       S.ym[kT3y + 3][tx], S.ym[kT3y + 2][tx], S.ym[kT3y + 1][tx], kd,
                                        S.c[kT3y + kT3h - 1][tx + kT3h], S.c[kT3y + kT3h][tx + kT3h]);
         }
       }
@@ -194,7 +193,7 @@ __device__ __forceinline__ void rk_sweep3d_body(const Args<float>& a, const Swee
                           S.zp[k & (kT3r - 1)][ty][tx], S.zp[(k + 1) & (kT3r - 1)][ty][tx],
                           S.zp[(k + 2) & (kT3r - 1)][ty][tx], S.zm[(k + 3) & (kT3r - 1)][ty][tx],
                           S.zm[(k + 2) & (kT3r - 1)][ty][tx], S.zm[(k + 1) & (kT3r - 1)][ty][tx],
-                          S.zm[k & (kT3r - 1)][ty][tx], S.zm[(k - 1) & (kT3r - 1)][ty][tx], alpha, kappa, chere,
+                          S.zm[k & (kT3r - 1)][ty][tx], S.zm[(k - 1) & (kT3r - 1)][ty][tx], kd, chere,
                           S.cz[(k + 1) & (kT3r - 1)][ty][tx]);
       }
     } else {
@@ -206,7 +205,7 @@ __device__ __forceinline__ void rk_sweep3d_body(const Args<float>& a, const Swee
           p[q] = P[q * st];
           m[q] = M[q * st];
         }
-        return face_flux_scheme<SCHEME>(p, m, alpha, kappa, cl, cr);
+        return face_flux_scheme<SCHEME>(p, m, kd, cl, cr);
       };
       if (!prime) {
         S.fx[ty][tx] =
@@ -228,7 +227,7 @@ __device__ __forceinline__ void rk_sweep3d_body(const Args<float>& a, const Swee
           p[q] = S.zp[(k - 2 + q) & (kT3r - 1)][ty][tx];
           m[q] = S.zm[(k - 2 + q) & (kT3r - 1)][ty][tx];
         }
-        fup = face_flux_scheme<SCHEME>(p, m, alpha, kappa, chere, S.cz[(k + 1) & (kT3r - 1)][ty][tx]);
+        fup = face_flux_scheme<SCHEME>(p, m, kd, chere, S.cz[(k + 1) & (kT3r - 1)][ty][tx]);
       }
     }
     __syncthreads();
@@ -236,19 +235,11 @@ __device__ __forceinline__ void rk_sweep3d_body(const Args<float>& a, const Swee
     // ---- divergence and the Shu-Osher combination of this stage
     if (!prime) {
       const float vs_floor = SUGAR && k == 0 ? a.vs * fmaf(-a.ks, __ldg(a.S + col), 1.f) : a.vs;
-      const float fdn = k == 0 ? -vs_floor * chere : carry;
-      const float L = S.fx[ty][tx] - S.fx[ty][tx + 1] + S.fy[ty][tx] - S.fy[ty + 1][tx] + fdn - fup;
+      const float Lk = S.fx[ty][tx] - S.fx[ty][tx + 1] + S.fy[ty][tx] - S.fy[ty + 1][tx] + carry - fup;
+      const float cb = k == 0 ? fmaf(-vs_floor, chere, chere) : chere;  // less the floor outflow (carry is 0 there)
       if (out) {
         const unsigned node = lv + col;
-        float v;
-        if (STAGE == 1) {
-          v = chere + L;
-        } else if (STAGE == 2) {
-          v = fmaf(0.75f, cn_here, 0.25f * (chere + L));
-        } else {
-          const float s = chere + L;
-          v = fmaf(1.f / 3.f, cn_here - s, s);
-        }
+        const float v = rk_combine<STAGE>(cb, Lk, alpha, cn_here);
         sp.cout[node] = v;
         if (STAGE == 3) report_status(a.status, !isfinite(v));
       }

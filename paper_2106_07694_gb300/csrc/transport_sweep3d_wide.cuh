@@ -17,7 +17,7 @@
 //    sweep;
 //  - the upper z face of each column comes from a private ring of the z-split fluxes of
 //    levels k-2 .. k+3, filled three levels ahead; the lower z face is carried.
-// Every face is computed once with the arithmetic of weno5_face_value/face_flux_x, so c is
+// Every face is computed once with the arithmetic of face_flux_x, so c is
 // bitwise that of the one-column kernel.
 //
 // Walls: ghost levels -2, -1, nz, nz+1 reflect c (even) and the fluid velocity (odd, Vs
@@ -25,7 +25,7 @@
 // its own kernel in 3D).
 #pragma once
 #include "common.cuh"
-#include "transport_sweep2d.cuh"       // weno5_q, weno5_face_value, face_flux_x
+#include "weno.cuh"
 #include "transport_sweep3d.cuh"       // Sweep3dParams
 #include "transport_stage2d_wide.cuh"  // lf_split
 
@@ -65,7 +65,7 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
   const unsigned X = (unsigned)(xl % nx), Y = (unsigned)(yl % ny);
   const unsigned plane = (unsigned)nx * (unsigned)ny, n = (unsigned)a.n;
   const unsigned col = Y * (unsigned)nx + X;
-  const float ia = a.inv_alpha, vs_a = a.vs * a.inv_alpha, alpha = a.alpha, kappa = a.kappa;
+  const float ia = a.inv_alpha, vs_a = a.vs * a.inv_alpha, alpha = a.alpha, kd = a.kappa * a.inv_alpha;
   const float* __restrict__ cin = sp.cin;
   const float* __restrict__ ux = a.u;
   const float* __restrict__ uy = a.u + n;
@@ -178,7 +178,7 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
         C[o] = __ldg(cin + lv + row + cx);
         lf_split(C[o], __ldg(ux + lv + row + cx) * ia, P[o], M[o]);
       }
-      S.xedge[h][w] = face_flux_x(P[0], P[1], P[2], P[3], P[4], M[5], M[4], M[3], M[2], M[1], alpha, kappa, C[2], C[3]);
+      S.xedge[h][w] = face_flux_x(P[0], P[1], P[2], P[3], P[4], M[5], M[4], M[3], M[2], M[1], kd, C[2], C[3]);
     } else {  // y face between rows y0 + kV3y - 1 and y0 + kV3y, tile column w - kV3y
       const int cl = w - kV3y;
       const unsigned cx = (unsigned)((x0 + cl) % nx);
@@ -189,7 +189,7 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
         lf_split(C[o], __ldg(uy + lv + row + cx) * ia, P[o], M[o]);
       }
       reinterpret_cast<float*>(&S.yedge[h][0])[cl] =
-          face_flux_x(P[0], P[1], P[2], P[3], P[4], M[5], M[4], M[3], M[2], M[1], alpha, kappa, C[2], C[3]);
+          face_flux_x(P[0], P[1], P[2], P[3], P[4], M[5], M[4], M[3], M[2], M[1], kd, C[2], C[3]);
     }
   }
 
@@ -243,11 +243,9 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
         }
 #pragma unroll
         for (int f = 0; f < 4; ++f) {
-          const float hp = fmaf(weno5_q(D[f], D[f + 1], D[f + 2], D[f + 3], SD[f], SD[f + 1], SD[f + 2]),
-                                1.f / 6.f, P[f + 2]);
-          const float hm = fmaf(weno5_q(-E[f + 3], -E[f + 2], -E[f + 1], -E[f], SE[f + 2], SE[f + 1], SE[f]),
-                                1.f / 6.f, M[f + 2]);
-          fxq[f] = fmaf(alpha, hp + hm, kappa * (C[f] - C[f + 1]));
+          const Recon<float> hp = weno5_recon(D[f], D[f + 1], D[f + 2], D[f + 3], SD[f], SD[f + 1], SD[f + 2]);
+          const Recon<float> hm = weno5_recon(-E[f + 3], -E[f + 2], -E[f + 1], -E[f], SE[f + 2], SE[f + 1], SE[f]);
+          fxq[f] = fmaf(kd, C[f] - C[f + 1], recon_sum(hp, P[f + 2], hm, M[f + 2]));
         }
         S.fx[b][ty][tx] = fxq[0];
         if (tx == kV3x - 1) S.fx[b][ty][kV3x] = S.xedge[k - z0][ty];
@@ -259,10 +257,10 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
         const float4 M1 = S.ym[sb][ty + 1][tx], M2 = S.ym[sb][ty + 2][tx], M3 = S.ym[sb][ty + 3][tx],
                      M4 = S.ym[sb][ty + 4][tx], M5 = S.ym[sb][ty + 5][tx];
         const float4 cb = S.c[sb][2 + ty][1 + tx];  // c of the row below
-        fyl.x = face_flux_x(P0.x, P1.x, P2.x, P3.x, P4.x, M5.x, M4.x, M3.x, M2.x, M1.x, alpha, kappa, cb.x, cq.x);
-        fyl.y = face_flux_x(P0.y, P1.y, P2.y, P3.y, P4.y, M5.y, M4.y, M3.y, M2.y, M1.y, alpha, kappa, cb.y, cq.y);
-        fyl.z = face_flux_x(P0.z, P1.z, P2.z, P3.z, P4.z, M5.z, M4.z, M3.z, M2.z, M1.z, alpha, kappa, cb.z, cq.z);
-        fyl.w = face_flux_x(P0.w, P1.w, P2.w, P3.w, P4.w, M5.w, M4.w, M3.w, M2.w, M1.w, alpha, kappa, cb.w, cq.w);
+        fyl.x = face_flux_x(P0.x, P1.x, P2.x, P3.x, P4.x, M5.x, M4.x, M3.x, M2.x, M1.x, kd, cb.x, cq.x);
+        fyl.y = face_flux_x(P0.y, P1.y, P2.y, P3.y, P4.y, M5.y, M4.y, M3.y, M2.y, M1.y, kd, cb.y, cq.y);
+        fyl.z = face_flux_x(P0.z, P1.z, P2.z, P3.z, P4.z, M5.z, M4.z, M3.z, M2.z, M1.z, kd, cb.z, cq.z);
+        fyl.w = face_flux_x(P0.w, P1.w, P2.w, P3.w, P4.w, M5.w, M4.w, M3.w, M2.w, M1.w, kd, cb.w, cq.w);
         S.fy[b][ty][tx] = fyl;
         if (ty == kV3y - 1) S.fy[b][kV3y][tx] = S.yedge[k - z0][tx];
       }
@@ -284,10 +282,10 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
                    P3 = S.zp[ring[3]][tid], P4 = S.zp[ring[4]][tid];
       const float4 M1 = S.zm[ring[1]][tid], M2 = S.zm[ring[2]][tid], M3 = S.zm[ring[3]][tid],
                    M4 = S.zm[ring[4]][tid], M5 = S.zm[ring[5]][tid];
-      fup[0] = face_flux_x(P0.x, P1.x, P2.x, P3.x, P4.x, M5.x, M4.x, M3.x, M2.x, M1.x, alpha, kappa, cq.x, cnext.x);
-      fup[1] = face_flux_x(P0.y, P1.y, P2.y, P3.y, P4.y, M5.y, M4.y, M3.y, M2.y, M1.y, alpha, kappa, cq.y, cnext.y);
-      fup[2] = face_flux_x(P0.z, P1.z, P2.z, P3.z, P4.z, M5.z, M4.z, M3.z, M2.z, M1.z, alpha, kappa, cq.z, cnext.z);
-      fup[3] = face_flux_x(P0.w, P1.w, P2.w, P3.w, P4.w, M5.w, M4.w, M3.w, M2.w, M1.w, alpha, kappa, cq.w, cnext.w);
+      fup[0] = face_flux_x(P0.x, P1.x, P2.x, P3.x, P4.x, M5.x, M4.x, M3.x, M2.x, M1.x, kd, cq.x, cnext.x);
+      fup[1] = face_flux_x(P0.y, P1.y, P2.y, P3.y, P4.y, M5.y, M4.y, M3.y, M2.y, M1.y, kd, cq.y, cnext.y);
+      fup[2] = face_flux_x(P0.z, P1.z, P2.z, P3.z, P4.z, M5.z, M4.z, M3.z, M2.z, M1.z, kd, cq.z, cnext.z);
+      fup[3] = face_flux_x(P0.w, P1.w, P2.w, P3.w, P4.w, M5.w, M4.w, M3.w, M2.w, M1.w, kd, cq.w, cnext.w);
     }
     // ring: level k + 4 replaces level k - 2; fetch level k + 5
     put_r(ring[0]);
@@ -307,20 +305,14 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
       const float ch[4] = {cq.x, cq.y, cq.z, cq.w};
       const float cnv[4] = {cn.x, cn.y, cn.z, cn.w};
       const float cy[4] = {carry.x, carry.y, carry.z, carry.w};
-      float v[4];
+      float v[4], cb[4] = {ch[0], ch[1], ch[2], ch[3]};
+      if (k == 0) {  // the floor row's settling outflow (its lower face, carry, is 0)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float fdn = k == 0 ? -a.vs * ch[j] : cy[j];
-        const float L = fxq[j] - fr[j] + fyl4[j] - fyu4[j] + fdn - fup[j];
-        if (STAGE == 1) {
-          v[j] = ch[j] + L;
-        } else if (STAGE == 2) {
-          v[j] = fmaf(0.75f, cnv[j], 0.25f * (ch[j] + L));
-        } else {
-          const float s = ch[j] + L;
-          v[j] = fmaf(1.f / 3.f, cnv[j] - s, s);
-        }
+        for (int j = 0; j < 4; ++j) cb[j] = fmaf(-a.vs, ch[j], ch[j]);
       }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        v[j] = rk_combine<STAGE>(cb[j], fxq[j] - fr[j] + fyl4[j] - fyu4[j] + cy[j] - fup[j], alpha, cnv[j]);
       if (out) {
         *reinterpret_cast<float4*>(sp.cout + (unsigned)k * plane + col) = make_float4(v[0], v[1], v[2], v[3]);
         if (STAGE == 3)
