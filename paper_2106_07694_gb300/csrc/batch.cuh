@@ -247,7 +247,7 @@ __device__ __forceinline__ void batch_stage_phase(const BatchTables& t, unsigned
     sp.cin = STAGE == 1 ? sa.c : (STAGE == 2 ? sa.c1 : sa.c2);
     sp.cout = STAGE == 1 ? sa.c1 : (STAGE == 2 ? sa.c2 : sa.c);
     sp.H = s_meta[4];
-    stage2d_wide_body<STAGE, LoadL2>(S, sa, sp, s_meta[1], s_meta[2], s_meta[3]);
+    stage2d_wide_body<STAGE, false, 0, LoadL2>(S, sa, sp, s_meta[1], s_meta[2], s_meta[3]);
     __syncthreads();
   }
   __syncthreads();

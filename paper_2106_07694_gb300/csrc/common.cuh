@@ -62,6 +62,15 @@ struct LoadPlain {
   static __device__ __forceinline__ float4 v4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 };
 
+// Four adjacent values (nx is a multiple of four and every field starts on a 256-byte line),
+// moved as one or two 16-byte accesses.
+template <typename T>
+struct alignas(4 * sizeof(T)) Quad {
+  T v[4];
+};
+template <typename T>
+__device__ __forceinline__ Quad<T> load_quad(const T* p) { return *reinterpret_cast<const Quad<T>*>(p); }
+
 constexpr int kSchemeWeno3 = 1;
 constexpr int kSchemeSignSplit = 2;
 
@@ -91,6 +100,28 @@ __device__ __forceinline__ int wrap_any(int a, int n) { return a < 0 ? a + n : (
 
 template <typename T>
 __device__ __forceinline__ bool finite_val(T v) { return isfinite(v); }
+
+// Sum of n FP64 partials written by other CTAs, by one whole warp in a fixed order (valid in
+// lane 0).  One thread that adds them in turn waits for a trip to L2 for each (sixteen took
+// 12 us), so up to eight are loaded together, and more are dealt to the lanes (l, l + 32, ...)
+// and folded by a shuffle tree, whose five FP64 steps cost about 1 us.
+__device__ __forceinline__ double fold_partials(const double* partials, int n) {
+  const volatile double* vp = partials;
+  double s = 0.0;
+  if (n <= 8) {
+    double v[8];
+#pragma unroll
+    for (int b = 0; b < 8; ++b) v[b] = b < n ? vp[b] : 0.0;
+#pragma unroll
+    for (int b = 0; b < 8; ++b)
+      if (b < n) s += v[b];
+    return s;
+  }
+  for (int b = (int)(threadIdx.x & 31); b < n; b += 32) s += vp[b];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  return s;
+}
 
 // Flag a bad value once per warp (no trap, no assert: the host reads the word).
 __device__ __forceinline__ unsigned lane_id() {

@@ -137,11 +137,11 @@ struct lbm_wenoc {
   lw::SweepLaunch sweep_geom{};
   bool sweep3d = false;  // 3D FP32 with walls: tiled z-sweep stage kernels
   int sweep3d_rows = 0;
-  bool wide3d = false;   // ... with four columns per thread (default scheme, no sugar)
+  bool wide3d = false;   // ... with four columns per thread (without LW_ONE_COLUMN)
   int wide3d_per_sm = 1;
   bool stage2d = false;  // 2D FP32 with walls: three row-sweep stage kernels
   int stage2d_rows = 0;
-  bool wide = false;     // ... with four columns per thread (default scheme, no sugar)
+  bool wide = false;     // ... with four columns per thread (FP32, without LW_ONE_COLUMN)
   int wide_per_sm = 1;   // CTAs of the four-column stage kernel one SM holds at once
   bool initialised = false;
   bool sugar = false;  // LW_SUGAR: S in L.sa / L.sb, selected by cur (the generic transport path)
@@ -167,6 +167,10 @@ struct lbm_wenoc {
 };
 
 namespace {
+
+int scheme_bits(const lbm_wenoc_params& p) {
+  return ((p.flags & LW_WENO3) ? lw::kSchemeWeno3 : 0) | ((p.flags & LW_SIGN_SPLIT) ? lw::kSchemeSignSplit : 0);
+}
 
 template <typename T>
 Args<T> make_args(const lbm_wenoc* h) {
@@ -196,7 +200,7 @@ Args<T> make_args(const lbm_wenoc* h) {
   a.alpha = T(h->alpha);
   a.inv_alpha = T(1.0 / h->alpha);
   a.u_cap = T(p.u_cap);
-  a.scheme = ((p.flags & LW_WENO3) ? lw::kSchemeWeno3 : 0) | ((p.flags & LW_SIGN_SPLIT) ? lw::kSchemeSignSplit : 0);
+  a.scheme = scheme_bits(p);
   if (h->sugar) {
     a.S = reinterpret_cast<T*>(b + (h->cur ? h->L.sb : h->L.sa));
     a.S2 = reinterpret_cast<T*>(b + (h->cur ? h->L.sa : h->L.sb));
@@ -281,8 +285,8 @@ void enqueue_transport(lbm_wenoc* h, const Args<T>& a);
 template <class LAT, typename T>
 void enqueue_sugar(lbm_wenoc* h, const Args<T>& a) {
   if (!h->sugar) return;
-  const dim3 blk(kLbmThreads);
-  const dim3 grd((a.nx + kLbmThreads - 1) / kLbmThreads, a.ny, a.nz);
+  const dim3 blk(lw::kSugarX, lw::kSugarY);
+  const dim3 grd(lw::sugar_blocks_x(a.nx) * (unsigned)(((long long)a.ny * a.nz + lw::kSugarY - 1) / lw::kSugarY));
   cudaStream_t s = h->stream;
   launch(h, K_SUGAR, [&] { lw::sugar_kernel<T, LAT::DIM><<<grd, blk, 0, s>>>(a); });
   h->cur ^= 1;
@@ -302,10 +306,10 @@ void enqueue_class_sum(lbm_wenoc* h) {
   lw::ClassPtrs<T> cp{};
   cp.count = h->ncls;
   for (int k = 0; k < h->ncls; ++k) cp.c[k] = class_ptr<T>(h, k);
-  const long long n = h->n;
+  const long long quads = h->n / 4;
   T* out = reinterpret_cast<T*>(h->ws + h->L.ctot);
   launch(h, K_OTHER, [&] {
-    lw::class_sum_kernel<T><<<(unsigned)((n + 255) / 256), 256, 0, h->stream>>>(cp, out, n);
+    lw::class_sum_kernel<T><<<(unsigned)((quads + 255) / 256), 256, 0, h->stream>>>(cp, out, quads);
   });
 }
 
@@ -361,7 +365,7 @@ void enqueue_transport(lbm_wenoc* h, const Args<T>& a) {
   const dim3 grd((a.nx + kLbmThreads - 1) / kLbmThreads, a.ny, a.nz);
   cudaStream_t s = h->stream;
   const long long nfloor = (long long)a.nx * (LAT::DIM == 3 ? a.ny : 1);
-  const int dep_blocks = (int)std::min<long long>(lw::kMaxReduceBlocks, (nfloor + 4095) / 4096);
+  const int dep_blocks = (int)std::min<long long>(lw::kMaxReduceBlocks, (nfloor + 1023) / 1024);
   if (std::is_same<T, float>::value && LAT::DIM == 2 && h->sweep) {
     const Args<float>& af = reinterpret_cast<const Args<float>&>(a);
     float* c_out = reinterpret_cast<float*>(h->ws + (h->cur ? h->L.c : h->L.c1));
@@ -552,6 +556,7 @@ int lbm_wenoc_create(const lbm_wenoc_params* p, void* dev_workspace, size_t byte
   h->frozen = (p->flags & LW_FROZEN_VELOCITY) != 0;
   h->sugar = (p->flags & LW_SUGAR) != 0;
   const bool variant = (p->flags & (LW_WENO3 | LW_SIGN_SPLIT)) != 0;  // transport-scheme variant
+  const int scheme = scheme_bits(*p);
   h->use_graphs = (p->flags & LW_NO_GRAPH) == 0;
   h->n = (long long)p->nx * p->ny * (p->dim == 3 ? p->nz : 1);
   h->ncls = classes_of(*p);
@@ -567,13 +572,13 @@ int lbm_wenoc_create(const lbm_wenoc_params* p, void* dev_workspace, size_t byte
   // the row-sweep stage kernels take the scheme variants and the sugar scalar too
   // (FP64 too: the validation build runs the one-column form)
   h->stage2d = h->p.dim == 2 && h->walls && !h->sweep && (p->nx + lw::kS2T - 1) / lw::kS2T <= lw::kMaxReduceBlocks;
-  h->wide = h->stage2d && !h->fp64 && !h->sugar && !variant && !(p->flags & LW_ONE_COLUMN);
+  h->wide = h->stage2d && !h->fp64 && !(p->flags & LW_ONE_COLUMN);
   if (h->stage2d) {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess || sms <= 0) sms = 148;
     if (h->wide) {
       int per_sm = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lw::rk_stage2d_wide_kernel<3>, lw::kWT, 0) !=
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lw::stage2d_wide_entry<3>(h->sugar, scheme), lw::kWT, 0) !=
               cudaSuccess ||
           per_sm <= 0)
         per_sm = 1;
@@ -597,14 +602,14 @@ int lbm_wenoc_create(const lbm_wenoc_params* p, void* dev_workspace, size_t byte
   if (h->sweep3d) {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess || sms <= 0) sms = 148;
-    h->wide3d = !h->sugar && !variant && !(p->flags & LW_ONE_COLUMN);
-    if (lw::sweep3d_prepare() != cudaSuccess || (h->wide3d && lw::sweep3d_wide_prepare() != cudaSuccess)) {
+    h->wide3d = !(p->flags & LW_ONE_COLUMN);
+    if ((h->wide3d ? lw::sweep3d_wide_prepare(h->sugar, scheme) : lw::sweep3d_prepare()) != cudaSuccess) {
       delete h;
       return LW_ECUDA;
     }
     if (h->wide3d) {
       int per_sm = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lw::rk_sweep3d_wide_kernel<3>, lw::kV3T,
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lw::sweep3d_wide_entry<3>(h->sugar, scheme), lw::kV3T,
                                                         lw::sweep3d_wide_smem()) != cudaSuccess ||
           per_sm <= 0)
         per_sm = 1;

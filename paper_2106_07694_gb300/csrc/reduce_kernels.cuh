@@ -1,8 +1,8 @@
 // FP64 reductions: the floor deposit of one step (a9) and the total mass.
 //
 // Deterministic: each block sums a fixed slice in a fixed tree order into
-// partials[block]; the block that takes the last ticket sums the partials in index
-// order and resets the ticket.  No floating-point atomics.
+// partials[block]; a warp of the block that takes the last ticket folds the partials
+// (fold_partials) and resets the ticket.  No floating-point atomics.
 #pragma once
 #include "common.cuh"
 
@@ -35,13 +35,13 @@ __device__ __forceinline__ void finish_reduction(double block_total, double* par
     last = (t == gridDim.x - 1);
   }
   __syncthreads();
-  if (last && threadIdx.x == 0) {
+  if (last && threadIdx.x < 32) {
     __threadfence();
-    double s = 0.0;
-    const volatile double* vp = partials;
-    for (unsigned b = 0; b < gridDim.x; ++b) s += vp[b];
-    *target = accumulate ? *target + s : s;
-    *ticket = 0u;
+    const double s = fold_partials(partials, (int)gridDim.x);
+    if (threadIdx.x == 0) {
+      *target = accumulate ? *target + s : s;
+      *ticket = 0u;
+    }
   }
 }
 
@@ -81,19 +81,22 @@ struct ClassPtrs {
 };
 
 // The loads of every class are issued before the sums (unrolled to the 8-class maximum);
-// the sum runs in class order.
+// the sum runs in class order, four nodes per thread.
 template <typename T>
-__global__ void class_sum_kernel(ClassPtrs<T> cp, T* out, long long n) {
+__global__ void class_sum_kernel(ClassPtrs<T> cp, T* out, long long quads) {
   const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  T v[8];
+  if (k >= quads) return;
+  Quad<T> v[8];
 #pragma unroll
-  for (int m = 0; m < 8; ++m) v[m] = m < cp.count ? __ldg(cp.c[m] + k) : T(0);
-  T acc = v[0];
+  for (int m = 0; m < 8; ++m)
+    if (m < cp.count) v[m] = load_quad(cp.c[m] + 4 * k);
+  Quad<T> acc = v[0];
 #pragma unroll
   for (int m = 1; m < 8; ++m)
-    if (m < cp.count) acc += v[m];
-  out[k] = acc;
+    if (m < cp.count)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc.v[j] += v[m].v[j];
+  *reinterpret_cast<Quad<T>*>(out + 4 * k) = acc;
 }
 
 }  // namespace lw

@@ -198,39 +198,57 @@ __global__ void __launch_bounds__(128) rk_stage_kernel(Args<T> a) {
 // axis in the advective form of Supplement Eqs. S5 (u > 0: backward difference) and S6
 // (u < 0: forward difference), with the velocity of this step's fluid update, plus
 // central diffusion D_s; walls mirror S (Neumann).  Writes S2.
+// A thread takes four adjacent columns of a row: bound by memory (S and u in, S2 out, 16 B a
+// node in 2D), where one column per thread moved 4 bytes a request
+// (1024 x 2048: 14.3 -> 8.6 us, 256^3 73 -> 54 us, launch and event overheads included).
+constexpr int kSugarX = 32, kSugarY = 4;  // threads along x (quads) and rows per block
+
+__host__ __device__ __forceinline__ unsigned sugar_blocks_x(int nx) { return (unsigned)(nx / 4 + kSugarX - 1) / kSugarX; }
+
 template <typename T, int DIM>
-__global__ void __launch_bounds__(128) sugar_kernel(Args<T> a) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y, z = blockIdx.z;
+__global__ void __launch_bounds__(kSugarX * kSugarY) sugar_kernel(Args<T> a) {
   const int nx = a.nx, ny = a.ny, nz = a.nz;
-  if (x >= nx) return;
+  const unsigned gx = sugar_blocks_x(nx);  // blocks along x; every block in grid.x, which has no 65535 limit
+  const int x = 4 * (int)(blockIdx.x % gx * kSugarX + threadIdx.x);
+  const int row = (int)(blockIdx.x / gx * kSugarY + threadIdx.y);
+  if (x >= nx || row >= ny * nz) return;
+  const int z = DIM == 2 ? 0 : row / ny, y = row - z * ny;
   const bool walls = a.walls != 0;
   const unsigned n = (unsigned)a.n;  // Q n < 2^31 (checked at create)
-  const unsigned node = ((unsigned)z * (unsigned)ny + (unsigned)y) * (unsigned)nx + (unsigned)x;
-  // neighbour offsets along each axis: x (and y in 3D) periodic; the vertical axis wraps, or
-  // at a wall takes offset 0 (the ghost mirrors the boundary node: no flux through the wall)
-  int off_m[3] = {x == 0 ? nx - 1 : -1, 0, 0}, off_p[3] = {x == nx - 1 ? -(nx - 1) : 1, 0, 0};
+  const unsigned node = (unsigned)row * (unsigned)nx + (unsigned)x;
+  // neighbour rows along the other axes: y in 3D is periodic; the vertical axis wraps, or at a
+  // wall takes offset 0 (the ghost mirrors the boundary node: no flux through the wall)
+  int off_m[2] = {0, 0}, off_p[2] = {0, 0};
   if (DIM == 2) {
-    off_m[1] = y == 0 ? (walls ? 0 : (ny - 1) * nx) : -nx;
-    off_p[1] = y == ny - 1 ? (walls ? 0 : -(ny - 1) * nx) : nx;
+    off_m[0] = y == 0 ? (walls ? 0 : (ny - 1) * nx) : -nx;
+    off_p[0] = y == ny - 1 ? (walls ? 0 : -(ny - 1) * nx) : nx;
   } else {
     const int plane = nx * ny;
-    off_m[1] = y == 0 ? (ny - 1) * nx : -nx;
-    off_p[1] = y == ny - 1 ? -(ny - 1) * nx : nx;
-    off_m[2] = z == 0 ? (walls ? 0 : (nz - 1) * plane) : -plane;
-    off_p[2] = z == nz - 1 ? (walls ? 0 : -(nz - 1) * plane) : plane;
+    off_m[0] = y == 0 ? (ny - 1) * nx : -nx;
+    off_p[0] = y == ny - 1 ? -(ny - 1) * nx : nx;
+    off_m[1] = z == 0 ? (walls ? 0 : (nz - 1) * plane) : -plane;
+    off_p[1] = z == nz - 1 ? (walls ? 0 : -(nz - 1) * plane) : plane;
   }
-  const T s0 = a.S[node];
-  T next = s0;
+  const Quad<T> s0 = load_quad(a.S + node), ux = load_quad(a.u + node);
+  const T left = a.S[x == 0 ? node + (unsigned)(nx - 1) : node - 1u];
+  const T right = a.S[x + 4 == nx ? node - (unsigned)x : node + 4u];
+  const T sx[6] = {left, s0.v[0], s0.v[1], s0.v[2], s0.v[3], right};
+  Quad<T> next = s0;
+  auto add = [&](int j, T u, T sm, T sc, T sp) {
+    next.v[j] -= u > T(0) ? u * (sc - sm) : u * (sp - sc);
+    next.v[j] += a.Ds * (sp - T(2) * sc + sm);
+  };
 #pragma unroll
-  for (int d = 0; d < DIM; ++d) {
-    const T sm = a.S[(unsigned)((int)node + off_m[d])];
-    const T sp = a.S[(unsigned)((int)node + off_p[d])];
-    const T u = a.u[(unsigned)d * n + node];
-    next -= u > T(0) ? u * (s0 - sm) : u * (sp - s0);
-    next += a.Ds * (sp - T(2) * s0 + sm);
+  for (int j = 0; j < 4; ++j) add(j, ux.v[j], sx[j], sx[j + 1], sx[j + 2]);
+#pragma unroll
+  for (int d = 1; d < DIM; ++d) {
+    const Quad<T> sm = load_quad(a.S + (unsigned)((int)node + off_m[d - 1]));
+    const Quad<T> sp = load_quad(a.S + (unsigned)((int)node + off_p[d - 1]));
+    const Quad<T> u = load_quad(a.u + (unsigned)d * n + node);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) add(j, u.v[j], sm.v[j], s0.v[j], sp.v[j]);
   }
-  a.S2[node] = next;
+  *reinterpret_cast<Quad<T>*>(a.S2 + node) = next;
 }
 
 }  // namespace lw

@@ -222,13 +222,13 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
       last = atomicAdd(a.ticket, 1u) == (unsigned)strips - 1;
     }
     __syncthreads();
-    if (last && t == 0) {
+    if (last && t < 32) {
       __threadfence();
-      const volatile double* vp = a.partials;
-      double tot = 0.0;
-      for (int b = 0; b < strips; ++b) tot += vp[b];
-      a.scalars[0] += tot;
-      *a.ticket = 0u;
+      const double tot = fold_partials(a.partials, strips);
+      if (t == 0) {
+        a.scalars[0] += tot;
+        *a.ticket = 0u;
+      }
     }
   }
 }

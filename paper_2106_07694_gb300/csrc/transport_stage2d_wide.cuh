@@ -1,7 +1,9 @@
 // 2D FP32 transport with four adjacent columns per thread: one SSP-RK3 stage of the
 // WENO5 + diffusion + settling update of c (steps a4..a8; the stage-3 kernel also folds
-// the floor deposit, a9).  Default scheme (Lax-Friedrichs WENO5), no sugar; the scheme
-// variants and the sugar scalar keep the one-column kernel of transport_stage2d.cuh.
+// the floor deposit, a9).  The scheme variants and the sugar scalar are compile-time
+// forms of the same kernel; against one column per thread, which shares no differences between
+// faces, their steps take 122 -> 88 us (sugar, 1024 x 2048), 129 -> 92 (WENO3, 1536 x 2048) and
+// 136 -> 103 (sign split).
 //
 // A CTA of kWT threads owns a strip of kWW = 4 kWT columns and a segment of rows and
 // sweeps it upward.  At row k:
@@ -55,9 +57,99 @@ __device__ __forceinline__ void lf_split(float c, float w, float& p, float& m) {
   m = fmaf(w, h, -h);
 }
 
-// LD: the global-load policy (LoadNC for a launch of its own, LoadL2 inside a kernel
-// whose earlier phases wrote the fields).
-template <int STAGE, class LD = LoadNC>
+// The pair a scheme stages at one node from c and w / alpha: the Lax-Friedrichs halves, or
+// for the sign split w c / alpha and w / alpha (face_flux_scheme).
+template <int SCHEME>
+__device__ __forceinline__ void scheme_split(float c, float w, float& p, float& m) {
+  if (SCHEME & kSchemeSignSplit) {
+    p = w * c;
+    m = w;
+  } else {
+    lf_split(c, w, p, m);
+  }
+}
+
+// Left x faces (divided by alpha) of four adjacent columns x .. x+3 from the staged quads of
+// columns x-4 .. x+7 (p, m: the scheme's pair), c of column x-1 and of the four: the first and
+// second differences are shared between the faces.
+template <int SCHEME>
+__device__ __forceinline__ void x_faces(const float4& p0, const float4& p1, const float4& p2, const float4& m0,
+                                        const float4& m1, const float4& m2, float c0w, const float4& cq, float kd,
+                                        float (&fxq)[4]) {
+  const float C[5] = {c0w, cq.x, cq.y, cq.z, cq.w};  // c at columns x-1 .. x+3
+  if constexpr (SCHEME == 0) {
+    const float P[8] = {p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w, p2.x};  // h+ at columns x-3 .. x+4
+    const float M[8] = {m0.z, m0.w, m1.x, m1.y, m1.z, m1.w, m2.x, m2.y};  // h- at columns x-2 .. x+5
+    float D[7], E[7], SD[6], SE[6];
+#pragma unroll
+    for (int j = 0; j < 7; ++j) {
+      D[j] = P[j + 1] - P[j];
+      E[j] = M[j + 1] - M[j];
+    }
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      SD[j] = D[j + 1] - D[j];
+      SE[j] = E[j + 1] - E[j];
+    }
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {  // face between columns x - 1 + f and x + f
+      const Recon<float> hp = weno5_recon(D[f], D[f + 1], D[f + 2], D[f + 3], SD[f], SD[f + 1], SD[f + 2]);
+      const Recon<float> hm = weno5_recon(-E[f + 3], -E[f + 2], -E[f + 1], -E[f], SE[f + 2], SE[f + 1], SE[f]);
+      fxq[f] = fmaf(kd, C[f] - C[f + 1], recon_sum(hp, P[f + 2], hm, M[f + 2]));
+    }
+  } else if constexpr (SCHEME == kSchemeWeno3) {  // three values a half: h+ at x-2 .. x+3, h- at x-1 .. x+4
+    const float P[6] = {p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+    const float M[6] = {m0.w, m1.x, m1.y, m1.z, m1.w, m2.x};
+    float D[5], E[5], A[5], B[5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      D[j] = P[j + 1] - P[j];
+      E[j] = M[j + 1] - M[j];
+      A[j] = weno3_smooth(D[j]);
+      B[j] = weno3_smooth(E[j]);
+    }
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      const Recon<float> hp = weno3_recon(D[f], D[f + 1], A[f], A[f + 1]);
+      const Recon<float> hm = weno3_recon(-E[f + 1], -E[f], B[f + 1], B[f]);
+      fxq[f] = fmaf(kd, C[f] - C[f + 1], recon_sum(hp, P[f + 1], hm, M[f + 1]));
+    }
+  } else {  // sign split: w c at columns x-3 .. x+5, w at x-1 .. x+3
+    const float P[9] = {p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w, p2.x, p2.y};
+    const float W[5] = {m0.w, m1.x, m1.y, m1.z, m1.w};
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      const float p[6] = {P[f], P[f + 1], P[f + 2], P[f + 3], P[f + 4], P[f + 5]};
+      const float m[6] = {0.f, 0.f, W[f], W[f + 1], 0.f, 0.f};
+      fxq[f] = face_flux_scheme<SCHEME>(p, m, kd, C[f], C[f + 1]);
+    }
+  }
+}
+
+// Faces between the third and fourth of six stacked rows, of four columns: P[q], M[q] the
+// staged pairs of row q, cl and cr c of rows 2 and 3.
+template <int SCHEME>
+__device__ __forceinline__ float4 column_faces(const float4 (&P)[6], const float4 (&M)[6], float kd, const float4& cl,
+                                               const float4& cr) {
+  auto face = [&](auto get, float l, float r) {
+    float p[6], m[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      p[q] = get(P[q]);
+      m[q] = get(M[q]);
+    }
+    return face_flux_scheme<SCHEME>(p, m, kd, l, r);
+  };
+  return make_float4(face([](const float4& v) { return v.x; }, cl.x, cr.x),
+                     face([](const float4& v) { return v.y; }, cl.y, cr.y),
+                     face([](const float4& v) { return v.z; }, cl.z, cr.z),
+                     face([](const float4& v) { return v.w; }, cl.w, cr.w));
+}
+
+// SUGAR: the settling velocity of a node is Vs (1 - ks S).  SCHEME: transport-scheme variant
+// bits (face_flux_scheme).  LD: the global-load policy (LoadNC for a launch of its own, LoadL2
+// inside a kernel whose earlier phases wrote the fields).
+template <int STAGE, bool SUGAR = false, int SCHEME = 0, class LD = LoadNC>
 __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<float>& a, const Stage2dParams& sp,
                                                   int bx, int by, int strips) {
   const int t = threadIdx.x;
@@ -89,10 +181,10 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
   };
   auto put_quad = [&](int b, int q, const float4& c, const float4& u) {
     float4 p, m;
-    lf_split(c.x, u.x * ia, p.x, m.x);
-    lf_split(c.y, u.y * ia, p.y, m.y);
-    lf_split(c.z, u.z * ia, p.z, m.z);
-    lf_split(c.w, u.w * ia, p.w, m.w);
+    scheme_split<SCHEME>(c.x, u.x * ia, p.x, m.x);
+    scheme_split<SCHEME>(c.y, u.y * ia, p.y, m.y);
+    scheme_split<SCHEME>(c.z, u.z * ia, p.z, m.z);
+    scheme_split<SCHEME>(c.w, u.w * ia, p.w, m.w);
     S.xp[b][q] = p;
     S.xm[b][q] = m;
     S.xc[b][q] = c;
@@ -104,7 +196,7 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
 
   // own columns, ring row l (ghost rows reflect: c even, u_y odd); rows past the ones any
   // face reads are clamped into the lattice and never used
-  float4 Rc, Ru;
+  float4 Rc, Ru, Rs = make_float4(0.f, 0.f, 0.f, 0.f);
   bool Rg = false;
   auto fetch_r = [&](int l) {
     Rg = l < 0 || l >= ny;
@@ -113,6 +205,7 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
     const unsigned row = (unsigned)lr * (unsigned)nx;
     Rc = LD::v4(cin + row + X);
     Ru = LD::v4(uy + row + X);
+    if (SUGAR) Rs = LD::v4(a.S + row + X);
   };
   // ring entries are addressed by byte offset (slot * kWT + t) * 16, rotated as the sweep advances
   auto ring_at = [&](float4 (*arr)[kWT], unsigned off) -> float4& {
@@ -121,10 +214,11 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
   auto put_r = [&](unsigned off) {
     const float s = Rg ? -ia : ia;
     float4 p, m;
-    lf_split(Rc.x, fmaf(Ru.x, s, -vs_a), p.x, m.x);
-    lf_split(Rc.y, fmaf(Ru.y, s, -vs_a), p.y, m.y);
-    lf_split(Rc.z, fmaf(Ru.z, s, -vs_a), p.z, m.z);
-    lf_split(Rc.w, fmaf(Ru.w, s, -vs_a), p.w, m.w);
+    auto vsa = [&](float S_) { return SUGAR ? vs_a * fmaf(-a.ks, S_, 1.f) : vs_a; };
+    scheme_split<SCHEME>(Rc.x, fmaf(Ru.x, s, -vsa(Rs.x)), p.x, m.x);
+    scheme_split<SCHEME>(Rc.y, fmaf(Ru.y, s, -vsa(Rs.y)), p.y, m.y);
+    scheme_split<SCHEME>(Rc.z, fmaf(Ru.z, s, -vsa(Rs.z)), p.z, m.z);
+    scheme_split<SCHEME>(Rc.w, fmaf(Ru.w, s, -vsa(Rs.w)), p.w, m.w);
     ring_at(S.yp, off) = p;
     ring_at(S.ym, off) = m;
   };
@@ -132,13 +226,14 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
   const int kb = y0 == 0 ? 0 : y0 - 1;  // first row: y0, or the priming row below it
   // first loads: the six ring rows and row kb, all in flight together (one after the other
   // they cost a trip to memory each: the 256 x 512 step 20.4 -> 18.6 us, 1024 x 2048 84.0 -> 80.1)
-  float4 rc[kWring], ru[kWring];
+  float4 rc[kWring], ru[kWring], rs[kWring];
   bool rg[kWring];
 #pragma unroll
   for (int j = 0; j < kWring; ++j) {
     fetch_r(kb - 2 + j);
     rc[j] = Rc;
     ru[j] = Ru;
+    if (SUGAR) rs[j] = Rs;
     rg[j] = Rg;
   }
   fetch_x(kb);
@@ -152,11 +247,11 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
       float P[6], M[6], C[6];
 #pragma unroll
       for (int o = 0; o < 6; ++o) {
-        const unsigned col = (unsigned)((x0 + kWW - 3 + o) % nx);
+        const unsigned col = (unsigned)wrap_inc(x0 + kWW - 3 + o, nx);
         C[o] = LD::s(cin + row + col);
-        lf_split(C[o], LD::s(ux + row + col) * ia, P[o], M[o]);
+        scheme_split<SCHEME>(C[o], LD::s(ux + row + col) * ia, P[o], M[o]);
       }
-      e = face_flux_x(P[0], P[1], P[2], P[3], P[4], M[5], M[4], M[3], M[2], M[1], kd, C[2], C[3]);
+      e = face_flux_scheme<SCHEME>(P, M, kd, C[2], C[3]);
     }
     S.edge[r] = e;
   }
@@ -167,6 +262,7 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
     ring[j] = (unsigned)((j * kWT + t) * sizeof(float4));
     Rc = rc[j];
     Ru = ru[j];
+    if (SUGAR) Rs = rs[j];
     Rg = rg[j];
     put_r(ring[j]);
   }
@@ -200,26 +296,7 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
       const float4 p0 = S.xp[b][t], p1 = S.xp[b][t + 1], p2 = S.xp[b][t + 2];
       const float4 m0 = S.xm[b][t], m1 = S.xm[b][t + 1], m2 = S.xm[b][t + 2];
       const float c0w = S.xc[b][t].w;
-      const float P[8] = {p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w, p2.x};  // h+ at columns x-3 .. x+4
-      const float M[8] = {m0.z, m0.w, m1.x, m1.y, m1.z, m1.w, m2.x, m2.y};  // h- at columns x-2 .. x+5
-      const float C[5] = {c0w, cq.x, cq.y, cq.z, cq.w};                     // c at columns x-1 .. x+3
-      float D[7], E[7], SD[6], SE[6];
-#pragma unroll
-      for (int j = 0; j < 7; ++j) {
-        D[j] = P[j + 1] - P[j];
-        E[j] = M[j + 1] - M[j];
-      }
-#pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        SD[j] = D[j + 1] - D[j];
-        SE[j] = E[j + 1] - E[j];
-      }
-#pragma unroll
-      for (int f = 0; f < 4; ++f) {  // face between columns x - 1 + f and x + f
-        const Recon<float> hp = weno5_recon(D[f], D[f + 1], D[f + 2], D[f + 3], SD[f], SD[f + 1], SD[f + 2]);
-        const Recon<float> hm = weno5_recon(-E[f + 3], -E[f + 2], -E[f + 1], -E[f], SE[f + 2], SE[f + 1], SE[f]);
-        fxq[f] = fmaf(kd, C[f] - C[f + 1], recon_sum(hp, P[f + 2], hm, M[f + 2]));
-      }
+      x_faces<SCHEME>(p0, p1, p2, m0, m1, m2, c0w, cq, kd, fxq);
       S.fx[b][t] = fxq[0];
       if (t == kWT - 1) S.fx[b][kWT] = S.edge[k - y0];
     }
@@ -227,14 +304,17 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
     // ---- upper y face of each column (the lid face carries nothing)
     float fup[4] = {0.f, 0.f, 0.f, 0.f};
     if (k != ny - 1) {
-      const float4 P0 = ring_at(S.yp, ring[0]), P1 = ring_at(S.yp, ring[1]), P2 = ring_at(S.yp, ring[2]),
-                   P3 = ring_at(S.yp, ring[3]), P4 = ring_at(S.yp, ring[4]);
-      const float4 M1 = ring_at(S.ym, ring[1]), M2 = ring_at(S.ym, ring[2]), M3 = ring_at(S.ym, ring[3]),
-                   M4 = ring_at(S.ym, ring[4]), M5 = ring_at(S.ym, ring[5]);
-      fup[0] = face_flux_x(P0.x, P1.x, P2.x, P3.x, P4.x, M5.x, M4.x, M3.x, M2.x, M1.x, kd, cq.x, cnext.x);
-      fup[1] = face_flux_x(P0.y, P1.y, P2.y, P3.y, P4.y, M5.y, M4.y, M3.y, M2.y, M1.y, kd, cq.y, cnext.y);
-      fup[2] = face_flux_x(P0.z, P1.z, P2.z, P3.z, P4.z, M5.z, M4.z, M3.z, M2.z, M1.z, kd, cq.z, cnext.z);
-      fup[3] = face_flux_x(P0.w, P1.w, P2.w, P3.w, P4.w, M5.w, M4.w, M3.w, M2.w, M1.w, kd, cq.w, cnext.w);
+      float4 P[6], M[6];
+#pragma unroll
+      for (int q = 0; q < 6; ++q) {
+        P[q] = ring_at(S.yp, ring[q]);
+        M[q] = ring_at(S.ym, ring[q]);
+      }
+      const float4 fu = column_faces<SCHEME>(P, M, kd, cq, cnext);
+      fup[0] = fu.x;
+      fup[1] = fu.y;
+      fup[2] = fu.z;
+      fup[3] = fu.w;
     }
     // ---- ring: row k + 4 replaces row k - 2; fetch row k + 5
     put_r(ring[0]);
@@ -259,9 +339,17 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
       const float cnv[4] = {cn.x, cn.y, cn.z, cn.w};
       const float cy[4] = {carry.x, carry.y, carry.z, carry.w};
       float v[4], cb[4] = {ch[0], ch[1], ch[2], ch[3]};
+      float vsf[4] = {a.vs, a.vs, a.vs, a.vs};
       if (k == 0) {  // the floor row's settling outflow (its lower face, carry, is 0)
+        if (SUGAR) {
+          const float4 s0 = LD::v4(a.S + X);
+          vsf[0] *= fmaf(-a.ks, s0.x, 1.f);
+          vsf[1] *= fmaf(-a.ks, s0.y, 1.f);
+          vsf[2] *= fmaf(-a.ks, s0.z, 1.f);
+          vsf[3] *= fmaf(-a.ks, s0.w, 1.f);
+        }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) cb[j] = fmaf(-a.vs, ch[j], ch[j]);
+        for (int j = 0; j < 4; ++j) cb[j] = fmaf(-vsf[j], ch[j], ch[j]);
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j) v[j] = rk_combine<STAGE>(cb[j], fxq[j] - fr[j] + cy[j] - fup[j], alpha, cnv[j]);
@@ -273,8 +361,10 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
             const float4 c1 = LD::v4(a.c1 + X);
             const float c1v[4] = {c1.x, c1.y, c1.z, c1.w};
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-              dep += fma((double)cnv[j] + (double)c1v[j], 1.0 / 6.0, (double)ch[j] * (2.0 / 3.0));
+            for (int j = 0; j < 4; ++j) {
+              const double b_ = fma((double)cnv[j] + (double)c1v[j], 1.0 / 6.0, (double)ch[j] * (2.0 / 3.0));
+              dep += SUGAR ? b_ * (double)vsf[j] : b_;  // with sugar Vs(S) per node, else Vs once at the fold
+            }
           }
         }
       }
@@ -285,7 +375,7 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
   if (STAGE > 1) cp_async_wait<0>();
 
   // stage 3: the CTAs holding the floor row fold the deposit of this step (FP64, fixed
-  // order: warp shuffles, then the last CTA sums the per-CTA partials in strip order)
+  // order: warp shuffles, then a warp of the last CTA folds the per-CTA partials)
   if (STAGE == 3 && y0 == 0) {
     double v = dep;
 #pragma unroll
@@ -295,27 +385,52 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
     if (t == 0) {
       double s2 = 0.0;
       for (int w = 0; w < kWT / 32; ++w) s2 += S.red[w];
-      a.partials[bx] = s2 * (double)a.vs;
-      __threadfence();
-      S.last = atomicAdd(a.ticket, 1u) == (unsigned)strips - 1;
+      if (!SUGAR) s2 *= (double)a.vs;
+      S.last = strips > 1;
+      if (strips == 1) {  // nothing to wait for: no fence and ticket (2.5 us of a small lattice's step)
+        *reinterpret_cast<volatile double*>(a.scalars) += s2;
+      } else {
+        a.partials[bx] = s2;
+        __threadfence();
+        S.last = atomicAdd(a.ticket, 1u) == (unsigned)strips - 1;
+      }
     }
     __syncthreads();
-    if (S.last && t == 0) {
+    if (S.last && t < 32) {
       __threadfence();
-      const volatile double* vp = a.partials;
-      double tot = 0.0;
-      for (int s = 0; s < strips; ++s) tot += vp[s];
       const double prev = *reinterpret_cast<volatile double*>(a.scalars);  // written by earlier steps
-      a.scalars[0] = prev + tot;
-      *a.ticket = 0u;
+      const double tot = fold_partials(a.partials, strips);
+      if (t == 0) {
+        a.scalars[0] = prev + tot;
+        *a.ticket = 0u;
+      }
     }
   }
 }
 
-template <int STAGE>
+template <int STAGE, bool SUGAR = false, int SCHEME = 0>
 __global__ void __launch_bounds__(kWT, kWminB) rk_stage2d_wide_kernel(Args<float> a, Stage2dParams sp) {
   __shared__ __align__(16) StageWideSmem S;
-  stage2d_wide_body<STAGE>(S, a, sp, blockIdx.x, blockIdx.y, gridDim.x);
+  stage2d_wide_body<STAGE, SUGAR, SCHEME>(S, a, sp, blockIdx.x, blockIdx.y, gridDim.x);
+}
+
+using StageWideKernel = void (*)(Args<float>, Stage2dParams);
+
+// The stage kernel of the handle's sugar and transport scheme (runtime fields).
+template <int STAGE>
+inline StageWideKernel stage2d_wide_entry(bool sugar, int scheme) {
+  switch (scheme) {
+    case kSchemeWeno3:
+      return sugar ? rk_stage2d_wide_kernel<STAGE, true, kSchemeWeno3> : rk_stage2d_wide_kernel<STAGE, false, kSchemeWeno3>;
+    case kSchemeSignSplit:
+      return sugar ? rk_stage2d_wide_kernel<STAGE, true, kSchemeSignSplit>
+                   : rk_stage2d_wide_kernel<STAGE, false, kSchemeSignSplit>;
+    case kSchemeWeno3 | kSchemeSignSplit:
+      return sugar ? rk_stage2d_wide_kernel<STAGE, true, kSchemeWeno3 | kSchemeSignSplit>
+                   : rk_stage2d_wide_kernel<STAGE, false, kSchemeWeno3 | kSchemeSignSplit>;
+    default:
+      return sugar ? rk_stage2d_wide_kernel<STAGE, true> : rk_stage2d_wide_kernel<STAGE>;
+  }
 }
 
 // Rows per segment of the four-column kernel.  The CTAs of a launch run in waves of
@@ -348,7 +463,7 @@ inline cudaError_t launch_stage2d_wide(const Args<float>& a, const float* cin, f
   sp.cout = cout;
   sp.H = H;
   const dim3 grid((a.nx + kWW - 1) / kWW, (a.ny + H - 1) / H);
-  rk_stage2d_wide_kernel<STAGE><<<grid, kWT, 0, s>>>(a, sp);
+  stage2d_wide_entry<STAGE>(a.S != nullptr, a.scheme)<<<grid, kWT, 0, s>>>(a, sp);
   return cudaGetLastError();
 }
 

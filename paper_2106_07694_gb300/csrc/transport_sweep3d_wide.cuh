@@ -1,7 +1,7 @@
 // 3D FP32 transport with four adjacent x columns per thread: one SSP-RK3 stage of the
 // WENO5 + diffusion + settling update of c (steps a4..a8) as a tiled sweep along the
-// vertical axis z.  Default scheme (Lax-Friedrichs WENO5), no sugar; the scheme variants
-// and the sugar scalar keep the one-column kernel of transport_sweep3d.cuh.
+// vertical axis z.  The scheme variants and the sugar scalar are compile-time forms of the
+// same kernel.
 //
 // A CTA of kV3x x kV3y threads owns a tile of 4 kV3x x kV3y (x, y) columns and a segment
 // of z levels and sweeps it upward.  At level k:
@@ -27,7 +27,7 @@
 #include "common.cuh"
 #include "weno.cuh"
 #include "transport_sweep3d.cuh"       // Sweep3dParams
-#include "transport_stage2d_wide.cuh"  // lf_split
+#include "transport_stage2d_wide.cuh"  // scheme_split, x_faces, column_faces
 
 namespace lw {
 
@@ -54,7 +54,8 @@ struct Sweep3dWideSmem {
   float4 yedge[kV3maxH][kV3x];     // top-edge y faces of the tile columns at each level
 };
 
-template <int STAGE>
+// SUGAR, SCHEME: as in the 2D kernel (stage2d_wide_body).
+template <int STAGE, bool SUGAR = false, int SCHEME = 0>
 __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args<float>& a, const Sweep3dParams& sp) {
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kV3x + tx;
   const int nx = a.nx, ny = a.ny, nz = a.nz;
@@ -120,20 +121,20 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
         if (sl_x[s]) {
           const float4 u = pu[s];
           float4 p, m;
-          lf_split(c.x, u.x * ia, p.x, m.x);
-          lf_split(c.y, u.y * ia, p.y, m.y);
-          lf_split(c.z, u.z * ia, p.z, m.z);
-          lf_split(c.w, u.w * ia, p.w, m.w);
+          scheme_split<SCHEME>(c.x, u.x * ia, p.x, m.x);
+          scheme_split<SCHEME>(c.y, u.y * ia, p.y, m.y);
+          scheme_split<SCHEME>(c.z, u.z * ia, p.z, m.z);
+          scheme_split<SCHEME>(c.w, u.w * ia, p.w, m.w);
           S.xp[b][sl_r[s] - 3][sl_q[s]] = p;
           S.xm[b][sl_r[s] - 3][sl_q[s]] = m;
         }
         if (sl_y[s]) {
           const float4 u = pv[s];
           float4 p, m;
-          lf_split(c.x, u.x * ia, p.x, m.x);
-          lf_split(c.y, u.y * ia, p.y, m.y);
-          lf_split(c.z, u.z * ia, p.z, m.z);
-          lf_split(c.w, u.w * ia, p.w, m.w);
+          scheme_split<SCHEME>(c.x, u.x * ia, p.x, m.x);
+          scheme_split<SCHEME>(c.y, u.y * ia, p.y, m.y);
+          scheme_split<SCHEME>(c.z, u.z * ia, p.z, m.z);
+          scheme_split<SCHEME>(c.w, u.w * ia, p.w, m.w);
           S.yp[b][sl_r[s]][sl_q[s] - 1] = p;
           S.ym[b][sl_r[s]][sl_q[s] - 1] = m;
         }
@@ -143,7 +144,7 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
 
   // own columns, ring level l (ghost levels reflect: c even, u_z odd); levels past the
   // ones any face reads are clamped into the lattice and never used
-  float4 Rc, Ru;
+  float4 Rc, Ru, Rs = make_float4(0.f, 0.f, 0.f, 0.f);
   bool Rg = false;
   auto fetch_r = [&](int l) {
     Rg = l < 0 || l >= nz;
@@ -152,14 +153,16 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
     const unsigned k3 = (unsigned)lr * plane + col;
     Rc = LoadNC::v4(cin + k3);
     Ru = LoadNC::v4(uz + k3);
+    if (SUGAR) Rs = LoadNC::v4(a.S + k3);
   };
   auto put_r = [&](int slot) {
     const float s = Rg ? -ia : ia;
     float4 p, m;
-    lf_split(Rc.x, fmaf(Ru.x, s, -vs_a), p.x, m.x);
-    lf_split(Rc.y, fmaf(Ru.y, s, -vs_a), p.y, m.y);
-    lf_split(Rc.z, fmaf(Ru.z, s, -vs_a), p.z, m.z);
-    lf_split(Rc.w, fmaf(Ru.w, s, -vs_a), p.w, m.w);
+    auto vsa = [&](float S_) { return SUGAR ? vs_a * fmaf(-a.ks, S_, 1.f) : vs_a; };
+    scheme_split<SCHEME>(Rc.x, fmaf(Ru.x, s, -vsa(Rs.x)), p.x, m.x);
+    scheme_split<SCHEME>(Rc.y, fmaf(Ru.y, s, -vsa(Rs.y)), p.y, m.y);
+    scheme_split<SCHEME>(Rc.z, fmaf(Ru.z, s, -vsa(Rs.z)), p.z, m.z);
+    scheme_split<SCHEME>(Rc.w, fmaf(Ru.w, s, -vsa(Rs.w)), p.w, m.w);
     S.zp[slot][tid] = p;
     S.zm[slot][tid] = m;
   };
@@ -176,9 +179,9 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
       for (int o = 0; o < 6; ++o) {
         const unsigned cx = (unsigned)((x0 + kV3W - 3 + o) % nx);
         C[o] = __ldg(cin + lv + row + cx);
-        lf_split(C[o], __ldg(ux + lv + row + cx) * ia, P[o], M[o]);
+        scheme_split<SCHEME>(C[o], __ldg(ux + lv + row + cx) * ia, P[o], M[o]);
       }
-      S.xedge[h][w] = face_flux_x(P[0], P[1], P[2], P[3], P[4], M[5], M[4], M[3], M[2], M[1], kd, C[2], C[3]);
+      S.xedge[h][w] = face_flux_scheme<SCHEME>(P, M, kd, C[2], C[3]);
     } else {  // y face between rows y0 + kV3y - 1 and y0 + kV3y, tile column w - kV3y
       const int cl = w - kV3y;
       const unsigned cx = (unsigned)((x0 + cl) % nx);
@@ -186,10 +189,10 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
       for (int o = 0; o < 6; ++o) {
         const unsigned row = (unsigned)((y0 + kV3y - 3 + o) % ny) * (unsigned)nx;
         C[o] = __ldg(cin + lv + row + cx);
-        lf_split(C[o], __ldg(uy + lv + row + cx) * ia, P[o], M[o]);
+        scheme_split<SCHEME>(C[o], __ldg(uy + lv + row + cx) * ia, P[o], M[o]);
       }
       reinterpret_cast<float*>(&S.yedge[h][0])[cl] =
-          face_flux_x(P[0], P[1], P[2], P[3], P[4], M[5], M[4], M[3], M[2], M[1], kd, C[2], C[3]);
+          face_flux_scheme<SCHEME>(P, M, kd, C[2], C[3]);
     }
   }
 
@@ -227,40 +230,20 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
         const float4 p0 = S.xp[sb][ty][tx], p1 = S.xp[sb][ty][tx + 1], p2 = S.xp[sb][ty][tx + 2];
         const float4 m0 = S.xm[sb][ty][tx], m1 = S.xm[sb][ty][tx + 1], m2 = S.xm[sb][ty][tx + 2];
         const float c0w = S.c[sb][3 + ty][tx].w;
-        const float P[8] = {p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w, p2.x};
-        const float M[8] = {m0.z, m0.w, m1.x, m1.y, m1.z, m1.w, m2.x, m2.y};
-        const float C[5] = {c0w, cq.x, cq.y, cq.z, cq.w};
-        float D[7], E[7], SD[6], SE[6];
-#pragma unroll
-        for (int j = 0; j < 7; ++j) {
-          D[j] = P[j + 1] - P[j];
-          E[j] = M[j + 1] - M[j];
-        }
-#pragma unroll
-        for (int j = 0; j < 6; ++j) {
-          SD[j] = D[j + 1] - D[j];
-          SE[j] = E[j + 1] - E[j];
-        }
-#pragma unroll
-        for (int f = 0; f < 4; ++f) {
-          const Recon<float> hp = weno5_recon(D[f], D[f + 1], D[f + 2], D[f + 3], SD[f], SD[f + 1], SD[f + 2]);
-          const Recon<float> hm = weno5_recon(-E[f + 3], -E[f + 2], -E[f + 1], -E[f], SE[f + 2], SE[f + 1], SE[f]);
-          fxq[f] = fmaf(kd, C[f] - C[f + 1], recon_sum(hp, P[f + 2], hm, M[f + 2]));
-        }
+        x_faces<SCHEME>(p0, p1, p2, m0, m1, m2, c0w, cq, kd, fxq);
         S.fx[b][ty][tx] = fxq[0];
         if (tx == kV3x - 1) S.fx[b][ty][kV3x] = S.xedge[k - z0][ty];
       }
       // lower y face of each column: y-split rows ty-3 .. ty+2 (staged rows ty .. ty+5)
       {
-        const float4 P0 = S.yp[sb][ty][tx], P1 = S.yp[sb][ty + 1][tx], P2 = S.yp[sb][ty + 2][tx],
-                     P3 = S.yp[sb][ty + 3][tx], P4 = S.yp[sb][ty + 4][tx];
-        const float4 M1 = S.ym[sb][ty + 1][tx], M2 = S.ym[sb][ty + 2][tx], M3 = S.ym[sb][ty + 3][tx],
-                     M4 = S.ym[sb][ty + 4][tx], M5 = S.ym[sb][ty + 5][tx];
+        float4 P[6], M[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+          P[q] = S.yp[sb][ty + q][tx];
+          M[q] = S.ym[sb][ty + q][tx];
+        }
         const float4 cb = S.c[sb][2 + ty][1 + tx];  // c of the row below
-        fyl.x = face_flux_x(P0.x, P1.x, P2.x, P3.x, P4.x, M5.x, M4.x, M3.x, M2.x, M1.x, kd, cb.x, cq.x);
-        fyl.y = face_flux_x(P0.y, P1.y, P2.y, P3.y, P4.y, M5.y, M4.y, M3.y, M2.y, M1.y, kd, cb.y, cq.y);
-        fyl.z = face_flux_x(P0.z, P1.z, P2.z, P3.z, P4.z, M5.z, M4.z, M3.z, M2.z, M1.z, kd, cb.z, cq.z);
-        fyl.w = face_flux_x(P0.w, P1.w, P2.w, P3.w, P4.w, M5.w, M4.w, M3.w, M2.w, M1.w, kd, cb.w, cq.w);
+        fyl = column_faces<SCHEME>(P, M, kd, cb, cq);
         S.fy[b][ty][tx] = fyl;
         if (ty == kV3y - 1) S.fy[b][kV3y][tx] = S.yedge[k - z0][tx];
       }
@@ -278,14 +261,17 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
     float fup[4] = {0.f, 0.f, 0.f, 0.f};
     if (k != nz - 1) {
       const float4 cnext = S.c[sn][3 + ty][1 + tx];
-      const float4 P0 = S.zp[ring[0]][tid], P1 = S.zp[ring[1]][tid], P2 = S.zp[ring[2]][tid],
-                   P3 = S.zp[ring[3]][tid], P4 = S.zp[ring[4]][tid];
-      const float4 M1 = S.zm[ring[1]][tid], M2 = S.zm[ring[2]][tid], M3 = S.zm[ring[3]][tid],
-                   M4 = S.zm[ring[4]][tid], M5 = S.zm[ring[5]][tid];
-      fup[0] = face_flux_x(P0.x, P1.x, P2.x, P3.x, P4.x, M5.x, M4.x, M3.x, M2.x, M1.x, kd, cq.x, cnext.x);
-      fup[1] = face_flux_x(P0.y, P1.y, P2.y, P3.y, P4.y, M5.y, M4.y, M3.y, M2.y, M1.y, kd, cq.y, cnext.y);
-      fup[2] = face_flux_x(P0.z, P1.z, P2.z, P3.z, P4.z, M5.z, M4.z, M3.z, M2.z, M1.z, kd, cq.z, cnext.z);
-      fup[3] = face_flux_x(P0.w, P1.w, P2.w, P3.w, P4.w, M5.w, M4.w, M3.w, M2.w, M1.w, kd, cq.w, cnext.w);
+      float4 P[6], M[6];
+#pragma unroll
+      for (int q = 0; q < 6; ++q) {
+        P[q] = S.zp[ring[q]][tid];
+        M[q] = S.zm[ring[q]][tid];
+      }
+      const float4 fu = column_faces<SCHEME>(P, M, kd, cq, cnext);
+      fup[0] = fu.x;
+      fup[1] = fu.y;
+      fup[2] = fu.z;
+      fup[3] = fu.w;
     }
     // ring: level k + 4 replaces level k - 2; fetch level k + 5
     put_r(ring[0]);
@@ -306,9 +292,17 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
       const float cnv[4] = {cn.x, cn.y, cn.z, cn.w};
       const float cy[4] = {carry.x, carry.y, carry.z, carry.w};
       float v[4], cb[4] = {ch[0], ch[1], ch[2], ch[3]};
-      if (k == 0) {  // the floor row's settling outflow (its lower face, carry, is 0)
+      if (k == 0) {  // the floor level's settling outflow (its lower face, carry, is 0)
+        float vsf[4] = {a.vs, a.vs, a.vs, a.vs};
+        if (SUGAR) {
+          const float4 s0 = LoadNC::v4(a.S + col);
+          vsf[0] *= fmaf(-a.ks, s0.x, 1.f);
+          vsf[1] *= fmaf(-a.ks, s0.y, 1.f);
+          vsf[2] *= fmaf(-a.ks, s0.z, 1.f);
+          vsf[3] *= fmaf(-a.ks, s0.w, 1.f);
+        }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) cb[j] = fmaf(-a.vs, ch[j], ch[j]);
+        for (int j = 0; j < 4; ++j) cb[j] = fmaf(-vsf[j], ch[j], ch[j]);
       }
 #pragma unroll
       for (int j = 0; j < 4; ++j)
@@ -324,20 +318,39 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
   }
 }
 
-template <int STAGE>
+template <int STAGE, bool SUGAR = false, int SCHEME = 0>
 __global__ void __launch_bounds__(kV3T, 4) rk_sweep3d_wide_kernel(Args<float> a, Sweep3dParams sp) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  sweep3d_wide_body<STAGE>(*reinterpret_cast<Sweep3dWideSmem*>(smem_raw), a, sp);
+  sweep3d_wide_body<STAGE, SUGAR, SCHEME>(*reinterpret_cast<Sweep3dWideSmem*>(smem_raw), a, sp);
+}
+
+using Sweep3dKernel = void (*)(Args<float>, Sweep3dParams);
+
+// The stage kernel of the handle's sugar and transport scheme (runtime fields).
+template <int STAGE>
+inline Sweep3dKernel sweep3d_wide_entry(bool sugar, int scheme) {
+  switch (scheme) {
+    case kSchemeWeno3:
+      return sugar ? rk_sweep3d_wide_kernel<STAGE, true, kSchemeWeno3> : rk_sweep3d_wide_kernel<STAGE, false, kSchemeWeno3>;
+    case kSchemeSignSplit:
+      return sugar ? rk_sweep3d_wide_kernel<STAGE, true, kSchemeSignSplit>
+                   : rk_sweep3d_wide_kernel<STAGE, false, kSchemeSignSplit>;
+    case kSchemeWeno3 | kSchemeSignSplit:
+      return sugar ? rk_sweep3d_wide_kernel<STAGE, true, kSchemeWeno3 | kSchemeSignSplit>
+                   : rk_sweep3d_wide_kernel<STAGE, false, kSchemeWeno3 | kSchemeSignSplit>;
+    default:
+      return sugar ? rk_sweep3d_wide_kernel<STAGE, true> : rk_sweep3d_wide_kernel<STAGE>;
+  }
 }
 
 inline size_t sweep3d_wide_smem() { return sizeof(Sweep3dWideSmem); }
 
-inline cudaError_t sweep3d_wide_prepare() {
+inline cudaError_t sweep3d_wide_prepare(bool sugar, int scheme) {
   const int bytes = (int)sizeof(Sweep3dWideSmem);
   const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(rk_sweep3d_wide_kernel<1>, at, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(rk_sweep3d_wide_kernel<2>, at, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(rk_sweep3d_wide_kernel<3>, at, bytes);
+  cudaError_t e = cudaFuncSetAttribute(sweep3d_wide_entry<1>(sugar, scheme), at, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(sweep3d_wide_entry<2>(sugar, scheme), at, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(sweep3d_wide_entry<3>(sugar, scheme), at, bytes);
   return e;
 }
 
@@ -370,7 +383,7 @@ inline cudaError_t launch_sweep3d_wide(const Args<float>& a, const float* cin, f
   sp.H = H;
   sp.ghost_shift = 2.f * a.vs * a.inv_alpha;
   const dim3 grid((a.nx + kV3W - 1) / kV3W, (a.ny + kV3y - 1) / kV3y, (a.nz + H - 1) / H);
-  rk_sweep3d_wide_kernel<STAGE><<<grid, dim3(kV3x, kV3y), sizeof(Sweep3dWideSmem), s>>>(a, sp);
+  sweep3d_wide_entry<STAGE>(a.S != nullptr, a.scheme)<<<grid, dim3(kV3x, kV3y), sizeof(Sweep3dWideSmem), s>>>(a, sp);
   return cudaGetLastError();
 }
 
