@@ -12,13 +12,18 @@
 //  - a thread reconstructs the left x faces of its four columns (first and second
 //    differences of the split fluxes shared between the four faces) and the lower y face
 //    of each of them; the x face right of its last column is its neighbour's first one,
-//    the y face above is the lower face of the thread above; for the tile's right column
-//    and top row these faces are computed for every level of the segment before the
-//    sweep;
+//    the y face above is the lower face of the thread above; the faces right of the tile's
+//    last column and above its top row come from the staged halo, by the first two warps
+//    (computed for the whole segment before the sweep, from global memory, they were nine
+//    trips to L2 before the first level and a tenth of the kernel);
 //  - the upper z face of each column comes from a private ring of the z-split fluxes of
 //    levels k-2 .. k+3, filled three levels ahead; the lower z face is carried.
 // Every face is computed once with the arithmetic of face_flux_x, so c is
 // bitwise that of the one-column kernel.
+//
+// Bound by instruction issue with 16 warps an SM (128 registers, 44.6 KB of shared memory a
+// CTA).  256 x 256 x 512: 391 / 388 / 411 us a stage, 476 / 476 / 491 with the edge faces ahead
+// of the sweep and the first loads one after the other.
 //
 // Walls: ghost levels -2, -1, nz, nz+1 reflect c (even) and the fluid velocity (odd, Vs
 // unchanged); the floor face carries -Vs c(0), the lid 0 (the floor deposit is folded by
@@ -37,21 +42,18 @@ constexpr int kV3T = kV3x * kV3y;       // threads per CTA
 constexpr int kV3W = 4 * kV3x;          // tile width in columns
 constexpr int kV3Qx = kV3x + 2;         // staged quads per row (tile and one halo quad per side)
 constexpr int kV3Ry = kV3y + 6;         // staged rows of the y stencil (three-row halo per side)
-constexpr int kV3maxH = 32;             // longest z segment (its edge faces are held in smem)
-constexpr int kV3Buf = 1;               // staging buffers: 1 (two barriers a level, four CTAs an SM)
+constexpr int kV3maxH = 32;             // longest z segment
 
 struct Sweep3dWideSmem {
-  float4 xp[kV3Buf][kV3y][kV3Qx];   // x-split h+/alpha of the tile rows (by level parity if two)
-  float4 xm[kV3Buf][kV3y][kV3Qx];
-  float4 yp[kV3Buf][kV3Ry][kV3x];   // y-split h+/alpha of the tile columns (rows -3 .. kV3y + 2)
-  float4 ym[kV3Buf][kV3Ry][kV3x];
-  float4 c[kV3Buf][kV3Ry][kV3Qx];   // stage input c (rows -3 .. kV3y + 2, quads -1 .. kV3x)
+  float4 xp[kV3y][kV3Qx];   // x-split h+/alpha of the tile rows
+  float4 xm[kV3y][kV3Qx];
+  float4 yp[kV3Ry][kV3x];   // y-split h+/alpha of the tile columns (rows -3 .. kV3y + 2)
+  float4 ym[kV3Ry][kV3x];
+  float4 c[kV3Ry][kV3Qx];   // stage input c (rows -3 .. kV3y + 2, quads -1 .. kV3x)
   float4 zp[6][kV3T];          // z-split ring of each thread's four columns
   float4 zm[6][kV3T];
   float fx[2][kV3y][kV3x + 1];     // first left x face of each thread (+ the tile's right edge)
   float4 fy[2][kV3y + 1][kV3x];    // lower y faces of each thread's columns (+ the tile's top edge)
-  float xedge[kV3maxH][kV3y];      // right-edge x face of each tile row at each level
-  float4 yedge[kV3maxH][kV3x];     // top-edge y faces of the tile columns at each level
 };
 
 // SUGAR, SCHEME: as in the 2D kernel (stage2d_wide_body).
@@ -112,12 +114,12 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
       }
     }
   };
-  auto stage_tile = [&](int b) {
+  auto stage_tile = [&]() {
 #pragma unroll
     for (int s = 0; s < kSl; ++s) {
       if (sl_on[s]) {
         const float4 c = pc[s];
-        S.c[b][sl_r[s]][sl_q[s]] = c;
+        S.c[sl_r[s]][sl_q[s]] = c;
         if (sl_x[s]) {
           const float4 u = pu[s];
           float4 p, m;
@@ -125,8 +127,8 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
           scheme_split<SCHEME>(c.y, u.y * ia, p.y, m.y);
           scheme_split<SCHEME>(c.z, u.z * ia, p.z, m.z);
           scheme_split<SCHEME>(c.w, u.w * ia, p.w, m.w);
-          S.xp[b][sl_r[s] - 3][sl_q[s]] = p;
-          S.xm[b][sl_r[s] - 3][sl_q[s]] = m;
+          S.xp[sl_r[s] - 3][sl_q[s]] = p;
+          S.xm[sl_r[s] - 3][sl_q[s]] = m;
         }
         if (sl_y[s]) {
           const float4 u = pv[s];
@@ -135,8 +137,8 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
           scheme_split<SCHEME>(c.y, u.y * ia, p.y, m.y);
           scheme_split<SCHEME>(c.z, u.z * ia, p.z, m.z);
           scheme_split<SCHEME>(c.w, u.w * ia, p.w, m.w);
-          S.yp[b][sl_r[s]][sl_q[s] - 1] = p;
-          S.ym[b][sl_r[s]][sl_q[s] - 1] = m;
+          S.yp[sl_r[s]][sl_q[s] - 1] = p;
+          S.ym[sl_r[s]][sl_q[s] - 1] = m;
         }
       }
     }
@@ -167,46 +169,33 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
     S.zm[slot][tid] = m;
   };
 
-  // edge faces of every level of the segment: right x edge of each tile row and top y edge
-  // of each tile column (the first faces of the neighbouring tiles)
-  for (int e = tid; e < (z1 - z0) * (kV3y + kV3W); e += kV3T) {
-    const int h = e / (kV3y + kV3W), w = e % (kV3y + kV3W);
-    const unsigned lv = (unsigned)(z0 + h) * plane;
-    float P[6], M[6], C[6];
-    if (w < kV3y) {  // x face between columns x0 + kV3W - 1 and x0 + kV3W, tile row w
-      const unsigned row = (unsigned)((y0 + w) % ny) * (unsigned)nx;
-#pragma unroll
-      for (int o = 0; o < 6; ++o) {
-        const unsigned cx = (unsigned)((x0 + kV3W - 3 + o) % nx);
-        C[o] = __ldg(cin + lv + row + cx);
-        scheme_split<SCHEME>(C[o], __ldg(ux + lv + row + cx) * ia, P[o], M[o]);
-      }
-      S.xedge[h][w] = face_flux_scheme<SCHEME>(P, M, kd, C[2], C[3]);
-    } else {  // y face between rows y0 + kV3y - 1 and y0 + kV3y, tile column w - kV3y
-      const int cl = w - kV3y;
-      const unsigned cx = (unsigned)((x0 + cl) % nx);
-#pragma unroll
-      for (int o = 0; o < 6; ++o) {
-        const unsigned row = (unsigned)((y0 + kV3y - 3 + o) % ny) * (unsigned)nx;
-        C[o] = __ldg(cin + lv + row + cx);
-        scheme_split<SCHEME>(C[o], __ldg(uy + lv + row + cx) * ia, P[o], M[o]);
-      }
-      reinterpret_cast<float*>(&S.yedge[h][0])[cl] =
-          face_flux_scheme<SCHEME>(P, M, kd, C[2], C[3]);
-    }
-  }
-
   const int kb = z0 == 0 ? 0 : z0 - 1;  // first level: z0, or the priming level below it
   int ring[6];                          // slots of levels k-2 .. k+3
+  {
+    // first loads: level kb of the tile and the six ring levels, all in flight together
+    float4 rc[6], ru[6], rs[6];
+    bool rg[6];
+    fetch_tile(kb);
 #pragma unroll
-  for (int j = 0; j < 6; ++j) {
-    ring[j] = j;
-    fetch_r(kb - 2 + j);
-    put_r(j);
+    for (int j = 0; j < 6; ++j) {
+      fetch_r(kb - 2 + j);
+      rc[j] = Rc;
+      ru[j] = Ru;
+      if (SUGAR) rs[j] = Rs;
+      rg[j] = Rg;
+    }
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      ring[j] = j;
+      Rc = rc[j];
+      Ru = ru[j];
+      if (SUGAR) Rs = rs[j];
+      Rg = rg[j];
+      put_r(j);
+    }
   }
   fetch_r(kb + 4);
-  fetch_tile(kb);
-  stage_tile(kV3Buf == 2 ? (kb & 1) : 0);
+  stage_tile();
   fetch_tile(kb + 1);  // kb + 1 <= z0 < nz
   float4 cn = make_float4(0.f, 0.f, 0.f, 0.f);
   if (STAGE > 1) cn = LoadNC::v4(a.c + (unsigned)kb * plane + col);
@@ -214,53 +203,71 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
   __syncthreads();
 
   for (int k = kb; k < z1; ++k) {
-    const int b = k & 1;                           // face exchange buffers
-    const int sb = kV3Buf == 2 ? b : 0;            // staging buffer of level k
-    const int sn = kV3Buf == 2 ? (b ^ 1) : 0;      // staging buffer of level k + 1
+    const int b = k & 1;  // face exchange buffers
     const bool prime = k < z0;
-    if (kV3Buf == 2 && k + 1 < nz) stage_tile(sn);  // level k + 1 (its c at the own columns: the z face)
-    if (kV3Buf == 2 && k + 1 < z1 && k + 2 < nz) fetch_tile(k + 2);
-    const float4 cq = S.c[sb][3 + ty][1 + tx];  // c of level k at this thread's columns
+    const float4 cq = S.c[3 + ty][1 + tx];  // c of level k at this thread's columns
 
     float fxq[4] = {0.f, 0.f, 0.f, 0.f};
     float4 fyl = make_float4(0.f, 0.f, 0.f, 0.f);
     if (!prime) {
       // left x faces of the four columns (shared differences, as in the 2D kernel)
       {
-        const float4 p0 = S.xp[sb][ty][tx], p1 = S.xp[sb][ty][tx + 1], p2 = S.xp[sb][ty][tx + 2];
-        const float4 m0 = S.xm[sb][ty][tx], m1 = S.xm[sb][ty][tx + 1], m2 = S.xm[sb][ty][tx + 2];
-        const float c0w = S.c[sb][3 + ty][tx].w;
+        const float4 p0 = S.xp[ty][tx], p1 = S.xp[ty][tx + 1], p2 = S.xp[ty][tx + 2];
+        const float4 m0 = S.xm[ty][tx], m1 = S.xm[ty][tx + 1], m2 = S.xm[ty][tx + 2];
+        const float c0w = S.c[3 + ty][tx].w;
         x_faces<SCHEME>(p0, p1, p2, m0, m1, m2, c0w, cq, kd, fxq);
         S.fx[b][ty][tx] = fxq[0];
-        if (tx == kV3x - 1) S.fx[b][ty][kV3x] = S.xedge[k - z0][ty];
       }
       // lower y face of each column: y-split rows ty-3 .. ty+2 (staged rows ty .. ty+5)
       {
         float4 P[6], M[6];
 #pragma unroll
         for (int q = 0; q < 6; ++q) {
-          P[q] = S.yp[sb][ty + q][tx];
-          M[q] = S.ym[sb][ty + q][tx];
+          P[q] = S.yp[ty + q][tx];
+          M[q] = S.ym[ty + q][tx];
         }
-        const float4 cb = S.c[sb][2 + ty][1 + tx];  // c of the row below
+        const float4 cb = S.c[2 + ty][1 + tx];  // c of the row below
         fyl = column_faces<SCHEME>(P, M, kd, cb, cq);
         S.fy[b][ty][tx] = fyl;
-        if (ty == kV3y - 1) S.fy[b][kV3y][tx] = S.yedge[k - z0][tx];
+      }
+      // the tile's top y faces (warp 0, a column each) and right x faces (warp 1, a row each)
+      if (tid < kV3W) {
+        const float* P = reinterpret_cast<const float*>(&S.yp[kV3y][0]) + tid;
+        const float* M = reinterpret_cast<const float*>(&S.ym[kV3y][0]) + tid;
+        const float* C = reinterpret_cast<const float*>(&S.c[kV3y + 2][1]) + tid;
+        float p[6], m[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+          p[q] = P[q * kV3W];
+          m[q] = M[q * kV3W];
+        }
+        reinterpret_cast<float*>(&S.fy[b][kV3y][0])[tid] = face_flux_scheme<SCHEME>(p, m, kd, C[0], C[4 * kV3Qx]);
+      } else if (tid < kV3W + kV3y) {
+        const int r = tid - kV3W;
+        const float* P = reinterpret_cast<const float*>(&S.xp[r][0]) + kV3W + 1;  // column kV3W - 3
+        const float* M = reinterpret_cast<const float*>(&S.xm[r][0]) + kV3W + 1;
+        const float* C = reinterpret_cast<const float*>(&S.c[3 + r][0]) + kV3W + 3;
+        float p[6], m[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+          p[q] = P[q];
+          m[q] = M[q];
+        }
+        S.fx[b][r][kV3x] = face_flux_scheme<SCHEME>(p, m, kd, C[0], C[1]);
       }
     }
 
     __syncthreads();
-    if (kV3Buf == 1) {  // one staging buffer: level k + 1 replaces level k once every face has read it
-      if (k + 1 < nz) stage_tile(0);
-      if (k + 1 < z1 && k + 2 < nz) fetch_tile(k + 2);
-      __syncthreads();
-    }
+    // one staging buffer: level k + 1 replaces level k once every face has read it
+    if (k + 1 < nz) stage_tile();
+    if (k + 1 < z1 && k + 2 < nz) fetch_tile(k + 2);
+    __syncthreads();
 
     // upper z face of each column from the ring (the lid face carries nothing); c of
     // level k + 1 at the own columns was staged before the barrier
     float fup[4] = {0.f, 0.f, 0.f, 0.f};
     if (k != nz - 1) {
-      const float4 cnext = S.c[sn][3 + ty][1 + tx];
+      const float4 cnext = S.c[3 + ty][1 + tx];
       float4 P[6], M[6];
 #pragma unroll
       for (int q = 0; q < 6; ++q) {
