@@ -6,12 +6,13 @@
 //   c1 = c + L(c; u); c2 = 3/4 c + 1/4 c1 + 1/4 L(c1; u); c' = 1/3 c + 2/3 c2 + 2/3 L(c2; u);
 //   J += Vs sum_floor(c/6 + c1/6 + 2 c2/3).
 // Given lambda(c') and lambda(g') and the recorded c, c1, c2, u, rho of the step, one
-// reverse step is six launches: the three transport stages backwards (for each,
-// adj_faces_kernel records every face's flux derivatives once and a gather sums, per node,
-// the records of the faces whose stencils contain it: the Jacobian-transpose of L with
-// respect to its input and to u, WENO5-JS nonlinear weights included), the last gather
-// fused with the fluid step backwards (reverse streaming with bounce-back, transpose of
-// the BGK-Guo collision, the velocity chain u = (j + F/2)/rho, the buoyancy F_y = -A c).
+// reverse step goes through the three transport stages backwards (the Jacobian-transpose of L
+// with respect to its input and to u, WENO5-JS nonlinear weights included), then the fluid
+// step backwards (reverse streaming with bounce-back, transpose of the BGK-Guo collision, the
+// velocity chain u = (j + F/2)/rho, the buoyancy F_y = -A c).  In FP32 a stage is one tile
+// kernel (adjoint_tile.cuh); in FP64 it is two launches: adj_faces_kernel records every face's
+// flux derivatives once and a gather sums, per node, the records of the faces whose stencils
+// contain it, the last gather fused with the fluid step.
 // The Lax-Friedrichs alpha is a fixed parameter here (the caller sets lf_alpha), so d/dVs
 // holds alpha fixed.  No atomics: results are bitwise reproducible and independent of the
 // checkpoint spacing.
@@ -369,24 +370,17 @@ __global__ void adj_vs_finish_kernel(const double* part, int nparts, double* out
   }
 }
 
-// Adjoint of the fluid step at one node, fused with the stage-1 gather (which completes
-// lambda(c^n)'s transport part lc and lambda(u) at this node).  Inputs: rho and u of step
-// n as the forward step computed them (recorded), c^n, lambda of the streamed populations
-// of step n+1 (natural layout lam_next[i][node]).  Outputs: lambda of the populations of
-// step n (natural layout) and lambda(c^n) = lc - A lambda(F_y) in mu.  The collision
-// g* = (1 - w) g + w geq(rho - 1, u) + src(u, F) and u = (j + F/2)/rho depend on the
+// Adjoint of the fluid step at one node.  Inputs: lc, gx, gy = the transport's lambda(c^n) and
+// lambda(u); rho and u of step n as the forward step computed them (recorded), c^n, lambda of
+// the streamed populations of step n+1 (natural layout lam_next[i][node]).  Outputs: lambda of
+// the populations of step n (natural layout) and lambda(c^n) = lc - A lambda(F_y) in mu.  The
+// collision g* = (1 - w) g + w geq(rho - 1, u) + src(u, F) and u = (j + F/2)/rho depend on the
 // populations only through rho and j.
 template <typename T>
-__global__ void __launch_bounds__(128) adj_gather_fluid_kernel(Args<T> a, AdjFields<T> f, FaceRecords<T> fr,
-                                                               const T* rho_rec, const T* lam_next, T* lam_out) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y;
-  if (x >= a.nx) return;
+__device__ __forceinline__ void adj_fluid_node(const Args<T>& a, const AdjFields<T>& f, const D2Q9Node& nd, T lc, T gx,
+                                               T gy, const T* rho_rec, const T* lam_next, T* lam_out) {
   const unsigned n = (unsigned)a.n;  // 24 n < 2^31 (checked by the host)
-  const D2Q9Node nd = d2q9_node(a, x, y);
   const unsigned node = nd.node;
-  T lc, gx, gy;
-  gather_node<T, 1>(a, f, fr, x, y, lc, gx, gy);
   const T Fx = a.bf[0], Fy = a.bf[1] - a.A * a.c[node];
   const T rho = rho_rec[node];
   const T ux = a.u[node], uy = a.u[n + node];
@@ -398,7 +392,7 @@ __global__ void __launch_bounds__(128) adj_gather_fluid_kernel(Args<T> a, AdjFie
   for (int i = 0; i < 9; ++i)
     mu[i] = nd.behind_wall(i, +1) ? lam_next[D2Q9::opp(i) * n + node]
                                   : lam_next[i * n + (unsigned)((int)node + nd.off(i, +1))];
-  T lam_drho = T(0), lux = f.lam_u[node] + gx, luy = f.lam_u[n + node] + gy, lFy = T(0);
+  T lam_drho = T(0), lux = gx, luy = gy, lFy = T(0);
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     const T wi = T(D2Q9::w(i));
@@ -422,6 +416,32 @@ __global__ void __launch_bounds__(128) adj_gather_fluid_kernel(Args<T> a, AdjFie
   for (int i = 0; i < 9; ++i)
     lam_out[i * n + node] = keep * mu[i] + lam_drho + ljx * T(D2Q9::cx(i)) + ljy * T(D2Q9::cy(i));
   f.mu[node] = lc - a.A * lFy;
+}
+
+// The same fused with the stage-1 gather of the recorded faces.
+template <typename T>
+__global__ void __launch_bounds__(128) adj_gather_fluid_kernel(Args<T> a, AdjFields<T> f, FaceRecords<T> fr,
+                                                               const T* rho_rec, const T* lam_next, T* lam_out) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int y = blockIdx.y;
+  if (x >= a.nx) return;
+  const D2Q9Node nd = d2q9_node(a, x, y);
+  T lc, gx, gy;
+  gather_node<T, 1>(a, f, fr, x, y, lc, gx, gy);
+  adj_fluid_node<T>(a, f, nd, lc, f.lam_u[nd.node] + gx, f.lam_u[(unsigned)a.n + nd.node] + gy, rho_rec, lam_next,
+                    lam_out);
+}
+
+// The same after the tile kernels (adjoint_tile.cuh), which leave lc and lambda(u) whole.
+template <typename T>
+__global__ void __launch_bounds__(128) adj_fluid_kernel(Args<T> a, AdjFields<T> f, const T* rho_rec, const T* lam_next,
+                                                        T* lam_out) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int y = blockIdx.y;
+  if (x >= a.nx) return;
+  const D2Q9Node nd = d2q9_node(a, x, y);
+  adj_fluid_node<T>(a, f, nd, f.lc[nd.node], f.lam_u[nd.node], f.lam_u[(unsigned)a.n + nd.node], rho_rec, lam_next,
+                    lam_out);
 }
 
 }  // namespace lw

@@ -26,6 +26,7 @@
 #include "transport_sweep3d_wide.cuh"
 #include "batch.cuh"
 #include "adjoint.cuh"
+#include "adjoint_tile.cuh"
 
 namespace {
 
@@ -278,7 +279,7 @@ void launch(lbm_wenoc* h, int kind, F&& f) {
 }
 
 template <class LAT, typename T>
-void enqueue_transport(lbm_wenoc* h, const Args<T>& a);
+void enqueue_transport(lbm_wenoc* h, const Args<T>& a, T* c_next);
 
 // Sugar: S^{n+1} from S^n and u^n into the other buffer (after the transport of c, which
 // reads S^n).
@@ -343,7 +344,7 @@ void enqueue_step(lbm_wenoc* h, int parity) {
     });
   }
   if (h->ncls == 1) {
-    enqueue_transport<LAT, T>(h, a);
+    enqueue_transport<LAT, T>(h, a, a.c);
   } else {
     // each class with its own settling velocity and deposit slot
     for (int k = 0; k < h->ncls; ++k) {
@@ -351,16 +352,17 @@ void enqueue_step(lbm_wenoc* h, int parity) {
       ak.c = class_ptr<T>(h, k);
       ak.vs = T(h->p.class_vs[k]);
       ak.scalars = a.scalars + kClassDeposit + k;
-      enqueue_transport<LAT, T>(h, ak);
+      enqueue_transport<LAT, T>(h, ak, ak.c);
     }
     enqueue_class_sum<T>(h);
   }
   enqueue_sugar<LAT, T>(h, a);
 }
 
-// The three RK stages (and the deposit) of one step on the fields a points at.
+// The three RK stages (and the deposit) of one step on the fields a points at; the new c goes
+// to c_next: a.c (in place), or with the 2D row-sweep stage kernels any other field.
 template <class LAT, typename T>
-void enqueue_transport(lbm_wenoc* h, const Args<T>& a) {
+void enqueue_transport(lbm_wenoc* h, const Args<T>& a, T* c_next) {
   const dim3 blk(kLbmThreads);
   const dim3 grd((a.nx + kLbmThreads - 1) / kLbmThreads, a.ny, a.nz);
   cudaStream_t s = h->stream;
@@ -379,13 +381,13 @@ void enqueue_transport(lbm_wenoc* h, const Args<T>& a) {
       const Args<float>& af = reinterpret_cast<const Args<float>&>(a);
       launch(h, K_STAGE1, [&] { lw::launch_stage2d_wide<1>(af, af.c, af.c1, H, s); });
       launch(h, K_STAGE2, [&] { lw::launch_stage2d_wide<2>(af, af.c1, af.c2, H, s); });
-      launch(h, K_STAGE3, [&] { lw::launch_stage2d_wide<3>(af, af.c2, af.c, H, s); });  // + deposit
+      launch(h, K_STAGE3, [&] { lw::launch_stage2d_wide<3>(af, af.c2, reinterpret_cast<float*>(c_next), H, s); });  // + deposit
       return;
     }
     // one column per thread, FP32 or FP64 (the validation build's 2D path)
     launch(h, K_STAGE1, [&] { lw::launch_stage2d<1, T>(a, a.c, a.c1, H, s); });
     launch(h, K_STAGE2, [&] { lw::launch_stage2d<2, T>(a, a.c1, a.c2, H, s); });
-    launch(h, K_STAGE3, [&] { lw::launch_stage2d<3, T>(a, a.c2, a.c, H, s); });  // + deposit
+    launch(h, K_STAGE3, [&] { lw::launch_stage2d<3, T>(a, a.c2, c_next, H, s); });  // + deposit
     return;
   }
   if (std::is_same<T, float>::value && LAT::DIM == 3 && h->sweep3d && h->wide3d) {
@@ -1530,7 +1532,7 @@ GradLayout grad_layout(const lbm_wenoc_params& p, int64_t nsteps, int32_t segmen
   G.vs = take(sizeof(double) * 4);
   G.nparts = ((p.nx + lw::kAdjThreads - 1) / lw::kAdjThreads) * p.ny;
   G.vs_part = take(sizeof(double) * (size_t)G.nparts);
-  G.faces = take(24 * n * es);
+  G.faces = take((p.flags & LW_FP64) ? 24 * n * es : 0);  // the FP32 tile kernels record no faces
   G.total = off;
   return G;
 }
@@ -1557,14 +1559,19 @@ StepRecord<T> step_record(unsigned char* aw, const GradLayout& G, int set, int64
   return R;
 }
 
-// One forward step that records what its adjoint needs: c^n is copied into the record,
-// and the step writes c1, c2, u and rho there instead of the handle's buffers.
+// One forward step that records what its adjoint needs: the step writes c1, c2, u and rho
+// into the record instead of the handle's buffers.  With the row-sweep stage kernels c^n is in
+// the record already (first: this is the segment's first step, which copies it there) and the
+// new c goes to the next step's record, or to the handle's buffer after the last one (next is
+// null); the one-node kernels update the handle's c in place, and c^n is copied each step.
 template <typename T>
-int record_step(lbm_wenoc* h, const StepRecord<T>& R) {
+int record_step(lbm_wenoc* h, const StepRecord<T>& R, bool first, T* next) {
   cudaStream_t s = h->stream;
   const size_t n = (size_t)h->n;
-  if (copy_d2d(R.c, h->ws + h->L.c, n * sizeof(T), s) != LW_OK) return LW_ECUDA;
+  if ((first || !h->stage2d) && copy_d2d(R.c, h->ws + h->L.c, n * sizeof(T), s) != LW_OK) return LW_ECUDA;
   Args<T> a = make_args<T>(h);
+  T* const c_own = a.c;
+  if (h->stage2d) a.c = R.c;
   a.c1 = R.c1;
   a.c2 = R.c2;
   a.u = R.u;
@@ -1575,7 +1582,7 @@ int record_step(lbm_wenoc* h, const StepRecord<T>& R) {
     else
       lw::lbm_d2q9_record_kernel<T, 1><<<grd, blk, 0, s>>>(a, R.rho);
   });
-  enqueue_transport<D2Q9, T>(h, a);
+  enqueue_transport<D2Q9, T>(h, a, h->stage2d && next ? next : c_own);
   h->parity ^= 1;
   h->steps += 1;
   return cudaGetLastError() == cudaSuccess ? LW_OK : LW_ECUDA;
@@ -1593,13 +1600,20 @@ int adjoint_step(lbm_wenoc* h, const StepRecord<T>& R, const lw::AdjFields<T>& f
   a.u = R.u;
   cudaStream_t s = h->stream;
   const dim3 blk(kLbmThreads), grd((a.nx + kLbmThreads - 1) / kLbmThreads, a.ny, 1);
-  launch(h, K_ADJ_FACES, [&] { lw::adj_faces_kernel<T, 3><<<grd, blk, 0, s>>>(a, f, fr); });
-  launch(h, K_ADJ_GATHER, [&] { lw::adj_gather_kernel<T, 3><<<grd, blk, 0, s>>>(a, f, fr); });
-  launch(h, K_ADJ_FACES, [&] { lw::adj_faces_kernel<T, 2><<<grd, blk, 0, s>>>(a, f, fr); });
-  launch(h, K_ADJ_GATHER, [&] { lw::adj_gather_kernel<T, 2><<<grd, blk, 0, s>>>(a, f, fr); });
-  launch(h, K_ADJ_FACES, [&] { lw::adj_faces_kernel<T, 1><<<grd, blk, 0, s>>>(a, f, fr); });
-  launch(h, K_ADJ_FLUID,
-         [&] { lw::adj_gather_fluid_kernel<T><<<grd, blk, 0, s>>>(a, f, fr, R.rho, lam_next, lam_out); });
+  if constexpr (std::is_same<T, float>::value) {  // a stage's faces and their gather in one tile kernel
+    launch(h, K_ADJ_FACES, [&] { lw::launch_adj_stage<3>(a, f, s); });
+    launch(h, K_ADJ_FACES, [&] { lw::launch_adj_stage<2>(a, f, s); });
+    launch(h, K_ADJ_FACES, [&] { lw::launch_adj_stage<1>(a, f, s); });
+    launch(h, K_ADJ_FLUID, [&] { lw::adj_fluid_kernel<T><<<grd, blk, 0, s>>>(a, f, R.rho, lam_next, lam_out); });
+  } else {
+    launch(h, K_ADJ_FACES, [&] { lw::adj_faces_kernel<T, 3><<<grd, blk, 0, s>>>(a, f, fr); });
+    launch(h, K_ADJ_GATHER, [&] { lw::adj_gather_kernel<T, 3><<<grd, blk, 0, s>>>(a, f, fr); });
+    launch(h, K_ADJ_FACES, [&] { lw::adj_faces_kernel<T, 2><<<grd, blk, 0, s>>>(a, f, fr); });
+    launch(h, K_ADJ_GATHER, [&] { lw::adj_gather_kernel<T, 2><<<grd, blk, 0, s>>>(a, f, fr); });
+    launch(h, K_ADJ_FACES, [&] { lw::adj_faces_kernel<T, 1><<<grd, blk, 0, s>>>(a, f, fr); });
+    launch(h, K_ADJ_FLUID,
+           [&] { lw::adj_gather_fluid_kernel<T><<<grd, blk, 0, s>>>(a, f, fr, R.rho, lam_next, lam_out); });
+  }
   return cudaGetLastError() == cudaSuccess ? LW_OK : LW_ECUDA;
 }
 
@@ -1639,6 +1653,7 @@ struct RecomputeStream {
 template <typename T>
 int deposit_gradient_impl(lbm_wenoc* h, const void* c0, int64_t nsteps, int32_t segment, unsigned char* aw,
                           const GradLayout& G, void* grad_c0, double* dJ_dVs, double* J) {
+  if (std::is_same<T, float>::value && lw::adj_stage_prepare() != cudaSuccess) return LW_ECUDA;
   int rc = lbm_wenoc_init(h, c0, nullptr);
   if (rc != LW_OK) return rc;
   cudaStream_t s = h->stream;
@@ -1648,8 +1663,10 @@ int deposit_gradient_impl(lbm_wenoc* h, const void* c0, int64_t nsteps, int32_t 
   auto seg_len = [&](int64_t sg) { return std::min<int64_t>(segment, nsteps - sg * segment); };
   auto set_of = [&](int64_t sg) { return G.rec_sets > 1 ? (int)(sg & 1) : 0; };
   auto record_segment = [&](int64_t sg) -> int {
-    for (int64_t k = 0; k < seg_len(sg); ++k) {
-      const int r = record_step<T>(h, step_record<T>(aw, G, set_of(sg), k));
+    const int64_t len = seg_len(sg);
+    for (int64_t k = 0; k < len; ++k) {
+      T* next = k + 1 < len ? step_record<T>(aw, G, set_of(sg), k + 1).c : nullptr;
+      const int r = record_step<T>(h, step_record<T>(aw, G, set_of(sg), k), k == 0, next);
       if (r != LW_OK) return r;
     }
     return LW_OK;
@@ -1731,7 +1748,7 @@ int deposit_gradient_impl(lbm_wenoc* h, const void* c0, int64_t nsteps, int32_t 
       break;
     }
     // the segment's reverse steps: replayed from a CUDA graph captured once per (record
-    // set, lambda buffer, length) -- six launches a step with no host gaps between them --
+    // set, lambda buffer, length) -- no host gaps between the launches of a step --
     // or launched one by one while the per-kernel timing is on
     const int64_t len = seg_len(sg);
     if (h->use_graphs && !h->profiling) {
@@ -1766,7 +1783,7 @@ int deposit_gradient_impl(lbm_wenoc* h, const void* c0, int64_t nsteps, int32_t 
         rc = LW_ECUDA;
         break;
       }
-      h->launches += 6 * len;
+      h->launches += (std::is_same<T, float>::value ? 4 : 6) * len;
       if (len & 1) cur ^= 1;
     } else {
       for (int64_t k = len - 1; k >= 0 && rc == LW_OK; --k) {
