@@ -24,6 +24,7 @@
 #include "transport_stage2d.cuh"
 #include "transport_stage2d_wide.cuh"
 #include "transport_sweep3d_wide.cuh"
+#include "transport_tile2d.cuh"
 #include "batch.cuh"
 #include "adjoint.cuh"
 #include "adjoint_tile.cuh"
@@ -143,6 +144,7 @@ struct lbm_wenoc {
   bool stage2d = false;  // 2D FP32 with walls: three row-sweep stage kernels
   int stage2d_rows = 0;
   bool wide = false;     // ... with four columns per thread (FP32, without LW_ONE_COLUMN)
+  bool tile = false;     // ... on tiles (four-column handles whose lattice stays in L2)
   int wide_per_sm = 1;   // CTAs of the four-column stage kernel one SM holds at once
   bool initialised = false;
   bool sugar = false;  // LW_SUGAR: S in L.sa / L.sb, selected by cur (the generic transport path)
@@ -377,6 +379,13 @@ void enqueue_transport(lbm_wenoc* h, const Args<T>& a, T* c_next) {
   }
   if (LAT::DIM == 2 && h->stage2d) {
     const int H = h->stage2d_rows;
+    if (std::is_same<T, float>::value && h->tile) {
+      const Args<float>& af = reinterpret_cast<const Args<float>&>(a);
+      launch(h, K_STAGE1, [&] { lw::launch_tile2d<1>(af, af.c, af.c1, s); });
+      launch(h, K_STAGE2, [&] { lw::launch_tile2d<2>(af, af.c1, af.c2, s); });
+      launch(h, K_STAGE3, [&] { lw::launch_tile2d<3>(af, af.c2, reinterpret_cast<float*>(c_next), s); });  // + deposit
+      return;
+    }
     if (std::is_same<T, float>::value && h->wide) {
       const Args<float>& af = reinterpret_cast<const Args<float>&>(a);
       launch(h, K_STAGE1, [&] { lw::launch_stage2d_wide<1>(af, af.c, af.c1, H, s); });
@@ -575,6 +584,7 @@ int lbm_wenoc_create(const lbm_wenoc_params* p, void* dev_workspace, size_t byte
   // (FP64 too: the validation build runs the one-column form)
   h->stage2d = h->p.dim == 2 && h->walls && !h->sweep && (p->nx + lw::kS2T - 1) / lw::kS2T <= lw::kMaxReduceBlocks;
   h->wide = h->stage2d && !h->fp64 && !(p->flags & LW_ONE_COLUMN);
+  h->tile = h->wide && lw::tile2d_use(p->nx, p->ny);
   if (h->stage2d) {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess || sms <= 0) sms = 148;

@@ -186,7 +186,7 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
     // ---- divergence and the Shu-Osher combination of this stage
     if (!prime) {
       const T vs_floor = SUGAR && k == 0 ? a.vs * fma_t(-a.ks, __ldg(a.S + X), T(1)) : a.vs;
-      const T Lk = S.fx[t] - S.fx[t + 1] + carry - fup;  // carry is 0 below the floor row
+      const T Lk = S.fx[t] - S.fx[t + 1] + (carry - fup);  // carry is 0 below the floor row
       const T cb = k == 0 ? fma_t(-vs_floor, chere, chere) : chere;  // less the floor outflow
       if (out) {
         const T v = rk_combine<STAGE>(cb, Lk, alpha, cn_here);

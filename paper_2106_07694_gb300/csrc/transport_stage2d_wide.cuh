@@ -50,6 +50,13 @@ struct StageWideSmem {
   bool last;
 };
 
+// Sum over eight neighbouring lanes (32 columns), valid in the first of each eight.
+__device__ __forceinline__ double tile_group_sum(double v) {
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // Lax-Friedrichs split of one node: p = h+/alpha, m = h-/alpha with h = c/2, w = u/alpha.
 __device__ __forceinline__ void lf_split(float c, float w, float& p, float& m) {
   const float h = 0.5f * c;
@@ -352,7 +359,7 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
         for (int j = 0; j < 4; ++j) cb[j] = fmaf(-vsf[j], ch[j], ch[j]);
       }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = rk_combine<STAGE>(cb[j], fxq[j] - fr[j] + cy[j] - fup[j], alpha, cnv[j]);
+      for (int j = 0; j < 4; ++j) v[j] = rk_combine<STAGE>(cb[j], fxq[j] - fr[j] + (cy[j] - fup[j]), alpha, cnv[j]);
       if (out) {
         *reinterpret_cast<float4*>(sp.cout + (unsigned)k * (unsigned)nx + X) = make_float4(v[0], v[1], v[2], v[3]);
         if (STAGE == 3) {
@@ -377,9 +384,9 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
   // stage 3: the CTAs holding the floor row fold the deposit of this step (FP64, fixed
   // order: warp shuffles, then a warp of the last CTA folds the per-CTA partials)
   if (STAGE == 3 && y0 == 0) {
-    double v = dep;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    double v = tile_group_sum(dep);
+    v += __shfl_down_sync(0xffffffffu, v, 8);
+    v += __shfl_down_sync(0xffffffffu, v, 16);
     if ((t & 31) == 0) S.red[t >> 5] = v;
     __syncthreads();
     if (t == 0) {
