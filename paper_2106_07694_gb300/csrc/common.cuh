@@ -40,6 +40,7 @@ struct Args {
   T ks;        // settling velocity Vs (1 - ks S)
   T Ds;        // sugar diffusivity
   int scheme;  // flux variant bits (kSchemeWeno3, kSchemeSignSplit); 0 = WENO5, Lax-Friedrichs
+  int late_count;  // deposit folded late (fold_late_deposit): partials a step's last stage leaves; 0 = it folds them
 };
 
 // Global-load policies.  LoadNC reads through the non-coherent (read-only) path, for data
@@ -121,6 +122,52 @@ __device__ __forceinline__ double fold_partials(const double* partials, int n) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   return s;
+}
+
+// The deposit's sums.  The four-column kernel adds the terms of 32 columns (eight threads), then
+// pairs of those groups twice (a warp), then its two warps, times Vs: a strip of 256 columns;
+// then the strips (fold_partials).  A tile holds one group; this fold, by a whole warp, rebuilds
+// the strips (valid in lane 0).
+__device__ __forceinline__ double fold_tile_partials(const double* partials, int tiles, double scale) {
+  const volatile double* vp = partials;
+  const int lane = threadIdx.x & 31, strips = (tiles + 7) / 8;
+  auto strip = [&](int b) {
+    double g[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) g[j] = 8 * b + j < tiles ? vp[8 * b + j] : 0.0;
+    return (((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7]))) * scale;
+  };
+  double s = 0.0;
+  if (strips <= 8) {
+    const double p = lane < strips ? strip(lane) : 0.0;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      const double v = __shfl_sync(0xffffffffu, p, b);
+      if (b < strips) s += v;
+    }
+    return s;
+  }
+  for (int b = lane; b < strips; b += 32) s += strip(b);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// Tile handles leave the fold of a step's deposit to the next kernel that can take it: the next
+// step's first stage (a block of its own, started first), or late_deposit_kernel before the
+// deposit is read.  The last stage then ends with one store a tile instead of a fence, a ticket
+// and a fold on its critical path (a step on 128 x 256 13.4 -> 11.3 us).  In the fluid kernel
+// the extra row of blocks cost more than that on lattices beyond L2 (108 -> 114 us on 2048 x 4096
+// in front of the lattice, 110 behind it).  The partials have a place of their own behind the
+// ones of the reductions that fold at once, and are zero before the first step and after
+// late_deposit_kernel, so adding them is always right.
+constexpr int kLateOffset = 512, kLateMax = 512;
+template <typename T>
+__device__ __forceinline__ void fold_late_deposit(const Args<T>& a) {
+  const double* p = a.partials + kLateOffset;
+  const double prev = *reinterpret_cast<const volatile double*>(a.scalars);
+  const double tot = fold_tile_partials(p, a.late_count, a.S ? 1.0 : (double)a.vs);
+  if ((threadIdx.x & 31) == 0) a.scalars[0] = prev + tot;
 }
 
 // Flag a bad value once per warp (no trap, no assert: the host reads the word).

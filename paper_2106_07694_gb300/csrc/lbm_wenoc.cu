@@ -145,6 +145,8 @@ struct lbm_wenoc {
   int stage2d_rows = 0;
   bool wide = false;     // ... with four columns per thread (FP32, without LW_ONE_COLUMN)
   bool tile = false;     // ... on tiles (four-column handles whose lattice stays in L2)
+  int late_count = 0;    // partials of the deposit folded late (0: the last stage folds them)
+  bool late_pending = false;  // a step since the last fold
   int wide_per_sm = 1;   // CTAs of the four-column stage kernel one SM holds at once
   bool initialised = false;
   bool sugar = false;  // LW_SUGAR: S in L.sa / L.sb, selected by cur (the generic transport path)
@@ -204,6 +206,7 @@ Args<T> make_args(const lbm_wenoc* h) {
   a.inv_alpha = T(1.0 / h->alpha);
   a.u_cap = T(p.u_cap);
   a.scheme = scheme_bits(p);
+  a.late_count = h->late_count;
   if (h->sugar) {
     a.S = reinterpret_cast<T*>(b + (h->cur ? h->L.sb : h->L.sa));
     a.S2 = reinterpret_cast<T*>(b + (h->cur ? h->L.sa : h->L.sb));
@@ -507,6 +510,22 @@ bool is_device_pointer(const void* p) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// Fold the deposit of the last step where that was left to the next one.
+int fold_late(lbm_wenoc* h) {
+  if (!h->late_pending) return LW_OK;
+  h->late_pending = false;
+  const Args<float> a = make_args<float>(h);  // FP32 handles only
+  lw::late_deposit_kernel<float><<<1, 32, 0, h->stream>>>(a);
+  return cudaGetLastError() == cudaSuccess ? LW_OK : LW_ECUDA;
+}
+
+// Partials, deposits and the status word of a fresh state (they lie one behind the other).
+int clear_reductions(lbm_wenoc* h) {
+  h->late_pending = false;
+  const size_t bytes = h->L.status + sizeof(unsigned) * 4 - h->L.partials;
+  return cudaMemsetAsync(h->ws + h->L.partials, 0, bytes, h->stream) == cudaSuccess ? LW_OK : LW_ECUDA;
+}
+
 template <class LAT, typename T>
 void launch_fields(lbm_wenoc* h, T* rho, T* u) {
   Args<T> a = make_args<T>(h);
@@ -631,6 +650,10 @@ int lbm_wenoc_create(const lbm_wenoc_params* p, void* dev_workspace, size_t byte
       h->sweep3d_rows = lw::sweep3d_rows(p->nx, p->ny, p->nz, sms, 0);
     }
   }
+  // on tiles the deposit of a step is folded by the next step (one class: the classes share the
+  // partials, one after the other)
+  if (h->tile && h->ncls == 1 && (p->nx + lw::kTX - 1) / lw::kTX <= lw::kLateMax)
+    h->late_count = (p->nx + lw::kTX - 1) / lw::kTX;
   h->kind_names.assign(kKindNames, kKindNames + K_COUNT);
   h->kind_launches.assign(K_COUNT, 0);
   h->kind_ms.assign(K_COUNT, 0.0);
@@ -655,9 +678,7 @@ int lbm_wenoc_init(lbm_wenoc* h, const void* c0, const void* u0) {
     if (cudaMemcpyAsync(h->ws + h->L.u, u0, ubytes, ku, h->stream) != cudaSuccess) return LW_ECUDA;
     u0dev = h->ws + h->L.u;
   }
-  if (cudaMemsetAsync(h->ws + h->L.scalars, 0, sizeof(double) * kScalars, h->stream) != cudaSuccess)
-    return LW_ECUDA;
-  if (cudaMemsetAsync(h->ws + h->L.status, 0, sizeof(unsigned) * 4, h->stream) != cudaSuccess) return LW_ECUDA;
+  if (clear_reductions(h) != LW_OK) return LW_ECUDA;
   if (h->sugar && cudaMemsetAsync(h->ws + h->L.sa, 0, cbytes, h->stream) != cudaSuccess) return LW_ECUDA;
   if (h->ncls > 1) {  // c0 is class 0; the others start empty, so phi_tot = c0
     if (cudaMemsetAsync(h->ws + h->L.cls, 0, h->L.ctot - h->L.cls, h->stream) != cudaSuccess) return LW_ECUDA;
@@ -692,6 +713,7 @@ int lbm_wenoc_step(lbm_wenoc* h, int64_t nsteps) {
   if (!h || nsteps < 0) return LW_EINVAL;
   if (!h->initialised) return LW_ESTATE;
   int64_t left = nsteps;
+  if (nsteps > 0) h->late_pending = h->late_count > 0;
   if (h->use_graphs && !h->profiling) {
     while (left > 0) {
       const int par = h->frozen ? 0 : h->parity;
@@ -730,7 +752,9 @@ int lbm_wenoc_step(lbm_wenoc* h, int64_t nsteps) {
 int lbm_wenoc_deposited_mass(lbm_wenoc* h, double* out) {
   if (!h || !out) return LW_EINVAL;
   if (!h->initialised) return LW_ESTATE;
-  int rc = sync_and_status(h);
+  int rc = fold_late(h);
+  if (rc != LW_OK) return rc;
+  rc = sync_and_status(h);
   if (rc == LW_ECUDA) return rc;
   if (h->ncls > 1) {
     double dep[kScalars];
@@ -751,7 +775,7 @@ static int sum_c(lbm_wenoc* h, long long count, double* out) {
     *out = 0.0;
     return LW_OK;
   }
-  const int blocks = (int)std::min<long long>(lw::kMaxReduceBlocks, (count + 8191) / 8192);
+  const int blocks = (int)std::min<long long>(lw::kLateOffset, (count + 8191) / 8192);  // the late partials lie behind
   const bool classes = h->ncls > 1;  // the sum of the classes
   if (h->fp64) {
     Args<double> a = make_args<double>(h);
@@ -901,6 +925,7 @@ int lbm_wenoc_save_state(lbm_wenoc* h, void* dst, size_t bytes) {
   if (!h->initialised) return LW_ESTATE;
   const size_t need = state_bytes(h);
   if (bytes < need) return LW_ENOMEM;
+  if (int rc = fold_late(h)) return rc;
   StateHeader hd{};
   hd.magic = kStateMagic;
   hd.version = kStateVersion;
@@ -939,6 +964,10 @@ int lbm_wenoc_load_state(lbm_wenoc* h, const void* src, size_t bytes) {
     off += align_up(r.bytes, 256);
   }
   if (cudaMemsetAsync(h->ws + h->L.status, 0, sizeof(unsigned) * 4, h->stream) != cudaSuccess) return LW_ECUDA;
+  // the loaded deposit is whole: nothing of an earlier step is left to fold
+  if (cudaMemsetAsync(h->ws + h->L.partials, 0, sizeof(double) * lw::kMaxReduceBlocks, h->stream) != cudaSuccess)
+    return LW_ECUDA;
+  h->late_pending = false;
   if (cudaStreamSynchronize(h->stream) != cudaSuccess) return LW_ECUDA;
   h->parity = hd.parity;
   h->steps = hd.steps;
@@ -1134,6 +1163,7 @@ int batch_upload_tables(lbm_wenoc_batch* b) {
   for (int i = 0; i < count; ++i) {
     lbm_wenoc* h = b->inst[i];
     args[i] = make_args<float>(h);
+    args[i].late_count = 0;  // the batch kernels' last stage folds its deposit itself
     lgx[i] = (h->p.nx + kLbmThreads - 1) / kLbmThreads;
     lstart[i + 1] = lstart[i] + lgx[i] * h->p.ny;
     sstrips[i] = (h->p.nx + lw::kWW - 1) / lw::kWW;
@@ -1253,6 +1283,7 @@ int batch_advance(lbm_wenoc_batch* b, int64_t nsteps, bool require_init) {
   for (lbm_wenoc* h : b->inst) {
     if (require_init && !h->initialised) return LW_ESTATE;
     if (h->parity != par || h->steps != b->inst[0]->steps) return LW_ESTATE;
+    if (int rc = fold_late(h)) return rc;  // of an instance stepped alone before
   }
   int64_t left = nsteps;
   int parity = par;
@@ -1288,9 +1319,7 @@ int batch_advance(lbm_wenoc_batch* b, int64_t nsteps, bool require_init) {
 int batch_trial_state(lbm_wenoc_batch* b) {
   for (lbm_wenoc* h : b->inst) {
     if (cudaMemsetAsync(h->ws + h->L.c, 0, (size_t)h->n * sizeof(float), b->stream) != cudaSuccess) return LW_ECUDA;
-    if (cudaMemsetAsync(h->ws + h->L.scalars, 0, sizeof(double) * kScalars, b->stream) != cudaSuccess)
-      return LW_ECUDA;
-    if (cudaMemsetAsync(h->ws + h->L.status, 0, sizeof(unsigned) * 4, b->stream) != cudaSuccess) return LW_ECUDA;
+    if (clear_reductions(h) != LW_OK) return LW_ECUDA;
     h->cur = 0;
     launch_init<D2Q9, float>(h, nullptr);
     h->parity = 0;
@@ -1585,6 +1614,7 @@ int record_step(lbm_wenoc* h, const StepRecord<T>& R, bool first, T* next) {
   a.c1 = R.c1;
   a.c2 = R.c2;
   a.u = R.u;
+  h->late_pending = h->late_count > 0;
   const dim3 blk(kLbmThreads), grd((a.nx + kLbmThreads - 1) / kLbmThreads, a.ny, 1);
   launch(h, K_LBM, [&] {
     if (h->parity == 0)

@@ -45,6 +45,14 @@ __device__ __forceinline__ void finish_reduction(double block_total, double* par
   }
 }
 
+// The late fold before the deposit is read (one warp); the partials are zero afterwards.
+template <typename T>
+__global__ void late_deposit_kernel(Args<T> a) {
+  fold_late_deposit(a);
+  __syncwarp();
+  for (int k = threadIdx.x; k < a.late_count; k += 32) a.partials[kLateOffset + k] = 0.0;
+}
+
 // a9: deposit += Vs * sum over the floor (v = 0) of c/6 + c1/6 + 2 c2/3 (RK3 b-weights,
 // so that sum c + deposit is invariant).  The floor is the first nfloor nodes.
 template <typename T>

@@ -393,8 +393,8 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
       double s2 = 0.0;
       for (int w = 0; w < kWT / 32; ++w) s2 += S.red[w];
       if (!SUGAR) s2 *= (double)a.vs;
-      S.last = strips > 1;
-      if (strips == 1) {  // nothing to wait for: no fence and ticket (2.5 us of a small lattice's step)
+      S.last = false;
+      if (strips == 1) {  // nothing to wait for: no fence and ticket
         *reinterpret_cast<volatile double*>(a.scalars) += s2;
       } else {
         a.partials[bx] = s2;

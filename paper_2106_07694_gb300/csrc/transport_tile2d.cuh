@@ -47,41 +47,19 @@ struct Tile2dSmem {
   float fx[kTY];             // right edge x face of each row
 };
 
-// The deposit's sums.  The four-column kernel adds the terms of 32 columns (eight threads), then
-// pairs of those groups twice (a warp), then its two warps, times Vs: a strip of 256 columns;
-// then the strips (fold_partials).  A tile holds one group; the fold rebuilds the strips.
-__device__ __forceinline__ double fold_tile_partials(const double* partials, int tiles, double scale) {
-  const volatile double* vp = partials;
-  const int lane = threadIdx.x & 31, strips = (tiles + 7) / 8;
-  auto strip = [&](int b) {
-    double g[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) g[j] = 8 * b + j < tiles ? vp[8 * b + j] : 0.0;
-    return (((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7]))) * scale;
-  };
-  double s = 0.0;
-  if (strips <= 8) {
-    const double p = lane < strips ? strip(lane) : 0.0;
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-      const double v = __shfl_sync(0xffffffffu, p, b);
-      if (b < strips) s += v;
-    }
-    return s;
-  }
-  for (int b = lane; b < strips; b += 32) s += strip(b);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-  return s;
-}
-
 template <int STAGE, bool SUGAR = false, int SCHEME = 0>
 __global__ void __launch_bounds__(kTT, 1024 / kTT) rk_tile2d_kernel(Args<float> a, Stage2dParams sp) {
   constexpr int TX = kTX, TY = kTY, T = kTT;
   __shared__ __align__(16) Tile2dSmem S;
   const int tid = threadIdx.x;
   const int nx = a.nx, ny = a.ny;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+  // the first stage's first row of blocks folds the deposit of the step before
+  const int by = (int)blockIdx.y - (STAGE == 1 && a.late_count > 0 ? 1 : 0);
+  if (STAGE == 1 && by < 0) {
+    if (blockIdx.x == 0 && tid < 32) fold_late_deposit(a);
+    return;
+  }
+  const int x0 = blockIdx.x * TX, y0 = by * TY;
   const float ia = a.inv_alpha, vs_a = a.vs * a.inv_alpha, alpha = a.alpha, kd = a.kappa * a.inv_alpha;
   const float* __restrict__ cin = sp.cin;
   const float* __restrict__ ux = a.u;
@@ -238,18 +216,20 @@ __global__ void __launch_bounds__(kTT, 1024 / kTT) rk_tile2d_kernel(Args<float> 
     }
   }
 
-  // stage 3: the floor tiles (their floor row is in the first eight threads) fold the deposit of
-  // this step: FP64, in the order of the four-column kernel
+  // stage 3: the floor tiles (their floor row is in the first eight threads) leave the deposit of
+  // this step for the next kernel, or fold it: FP64, in the order of the four-column kernel
   if (STAGE == 3 && y0 == 0 && tid < 32) {
     const double v = tile_group_sum(dep);
+    if (a.late_count > 0) {
+      if (tid == 0) a.partials[kLateOffset + blockIdx.x] = v;
+      return;
+    }
     const int tiles = gridDim.x;
-    int last = tiles == 1;
+    int last = 0;
     if (tid == 0) {
       a.partials[blockIdx.x] = v;
-      if (tiles > 1) {
-        __threadfence();
-        last = atomicAdd(a.ticket, 1u) == (unsigned)tiles - 1;
-      }
+      __threadfence();
+      last = atomicAdd(a.ticket, 1u) == (unsigned)tiles - 1;
     }
     if (__shfl_sync(0xffffffffu, last, 0)) {
       __threadfence();
@@ -289,7 +269,7 @@ inline cudaError_t launch_tile2d(const Args<float>& a, const float* cin, float* 
   sp.cin = cin;
   sp.cout = cout;
   sp.H = kTY;
-  const dim3 grid((a.nx + kTX - 1) / kTX, (a.ny + kTY - 1) / kTY);
+  const dim3 grid((a.nx + kTX - 1) / kTX, (a.ny + kTY - 1) / kTY + (STAGE == 1 && a.late_count > 0 ? 1 : 0));
   tile2d_entry<STAGE>(a.S != nullptr, a.scheme)<<<grid, kTT, 0, s>>>(a, sp);
   return cudaGetLastError();
 }
