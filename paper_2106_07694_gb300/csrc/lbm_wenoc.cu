@@ -492,13 +492,37 @@ int launches_per_step(const lbm_wenoc* h) {
 
 int64_t launches_for(const lbm_wenoc* h, int64_t count) { return (int64_t)launches_per_step(h) * count; }
 
-int sync_and_status(lbm_wenoc* h) {
-  if (cudaStreamSynchronize(h->stream) != cudaSuccess) return LW_ECUDA;
-  unsigned st[2] = {0, 0};
-  if (cudaMemcpy(st, h->ws + h->L.status, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess) return LW_ECUDA;
-  if (st[0] & lw::kStatusTimeout) return LW_ETIMEOUT;
-  if (st[0] & lw::kStatusUnstable) return LW_EUNSTABLE;
+// The scalars and the status word, which lie one behind the other: one copy and one wait for the
+// stream's work so far (a wait and a copy each cost a caller who reads the deposit and the mass
+// every few steps 117 us a pair).
+struct Readback {
+  double scalars[kScalars];
+  unsigned status;
+};
+
+int read_back(lbm_wenoc* h, Readback* r) {
+  const size_t bytes = h->L.status + sizeof(unsigned) - h->L.scalars;
+  unsigned char buf[512];
+  static_assert(sizeof(double) * kScalars + 256 + sizeof(unsigned) <= sizeof(buf), "scalars and status fit");
+  if (bytes > sizeof(buf)) return LW_ECUDA;
+  if (cudaMemcpyAsync(buf, h->ws + h->L.scalars, bytes, cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
+      cudaStreamSynchronize(h->stream) != cudaSuccess)
+    return LW_ECUDA;
+  std::memcpy(r->scalars, buf, sizeof(double) * kScalars);
+  std::memcpy(&r->status, buf + (h->L.status - h->L.scalars), sizeof(unsigned));
   return LW_OK;
+}
+
+int status_code(unsigned st) {
+  if (st & lw::kStatusTimeout) return LW_ETIMEOUT;
+  if (st & lw::kStatusUnstable) return LW_EUNSTABLE;
+  return LW_OK;
+}
+
+int sync_and_status(lbm_wenoc* h) {
+  Readback r;
+  const int rc = read_back(h, &r);
+  return rc != LW_OK ? rc : status_code(r.status);
 }
 
 bool is_device_pointer(const void* p) {
@@ -508,6 +532,19 @@ bool is_device_pointer(const void* p) {
     return false;
   }
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+}
+
+// A caller's buffer that a kernel of the handle may read or write itself: ordinary device memory
+// of the handle's device, aligned to its element.  Others (host memory, another device's, a
+// managed buffer) go through a copy.
+bool kernel_can_use(const lbm_wenoc* h, const void* p) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == h->device &&
+         reinterpret_cast<uintptr_t>(p) % (h->fp64 ? 8u : 4u) == 0;
 }
 
 // Fold the deposit of the last step where that was left to the next one.
@@ -672,8 +709,12 @@ int lbm_wenoc_init(lbm_wenoc* h, const void* c0, const void* u0) {
   cudaMemcpyKind kc = is_device_pointer(c0) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   if (cudaMemcpyAsync(h->ws + h->L.c, c0, cbytes, kc, h->stream) != cudaSuccess) return LW_ECUDA;
   const void* u0dev = nullptr;
-  if (u0) {
+  bool host_source = kc == cudaMemcpyHostToDevice;
+  if (u0 && kernel_can_use(h, u0)) {
+    u0dev = u0;  // read where it is
+  } else if (u0) {
     cudaMemcpyKind ku = is_device_pointer(u0) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+    host_source = host_source || ku == cudaMemcpyHostToDevice;
     // stage through the population buffer's tail is unsafe; use u itself then copy in kernel
     if (cudaMemcpyAsync(h->ws + h->L.u, u0, ubytes, ku, h->stream) != cudaSuccess) return LW_ECUDA;
     u0dev = h->ws + h->L.u;
@@ -699,7 +740,7 @@ int lbm_wenoc_init(lbm_wenoc* h, const void* c0, const void* u0) {
   }
   if (cudaGetLastError() != cudaSuccess) return LW_ECUDA;
   // host sources may be pageable: make the call safe to return
-  if (kc == cudaMemcpyHostToDevice || (u0 && !is_device_pointer(u0)))
+  if (host_source)
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return LW_ECUDA;
   h->parity = 0;
   h->cur = 0;
@@ -749,33 +790,31 @@ int lbm_wenoc_step(lbm_wenoc* h, int64_t nsteps) {
   return LW_OK;
 }
 
+// The accumulated deposit, of every class.
+static double total_deposit(const lbm_wenoc* h, const Readback& r) {
+  if (h->ncls == 1) return r.scalars[0];
+  double tot = 0.0;
+  for (int k = 0; k < h->ncls; ++k) tot += r.scalars[kClassDeposit + k];
+  return tot;
+}
+
 int lbm_wenoc_deposited_mass(lbm_wenoc* h, double* out) {
   if (!h || !out) return LW_EINVAL;
   if (!h->initialised) return LW_ESTATE;
   int rc = fold_late(h);
   if (rc != LW_OK) return rc;
-  rc = sync_and_status(h);
-  if (rc == LW_ECUDA) return rc;
-  if (h->ncls > 1) {
-    double dep[kScalars];
-    if (cudaMemcpy(dep, h->ws + h->L.scalars, sizeof(dep), cudaMemcpyDeviceToHost) != cudaSuccess) return LW_ECUDA;
-    double tot = 0.0;
-    for (int k = 0; k < h->ncls; ++k) tot += dep[kClassDeposit + k];
-    *out = tot;
-    return rc;
-  }
-  if (cudaMemcpy(out, h->ws + h->L.scalars, sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
-    return LW_ECUDA;
-  return rc;
+  Readback r;
+  if ((rc = read_back(h, &r)) != LW_OK) return rc;
+  *out = total_deposit(h, r);
+  return status_code(r.status);
 }
 
-// Sum of c (or of the classes) over the first `count` nodes, FP64 in a fixed order, into *out.
-static int sum_c(lbm_wenoc* h, long long count, double* out) {
-  if (count <= 0) {
-    *out = 0.0;
-    return LW_OK;
-  }
-  const int blocks = (int)std::min<long long>(lw::kLateOffset, (count + 8191) / 8192);  // the late partials lie behind
+// Enqueue the sum of c (or of the classes) over the first `count` nodes, FP64 in a fixed order,
+// into scalars[1].
+static int enqueue_sum_c(lbm_wenoc* h, long long count) {
+  // blocks of 1024 nodes while they last (one trip to memory a thread); the late partials lie
+  // behind the first kLateOffset
+  const int blocks = (int)std::min<long long>(lw::kLateOffset, (count + 1023) / 1024);
   const bool classes = h->ncls > 1;  // the sum of the classes
   if (h->fp64) {
     Args<double> a = make_args<double>(h);
@@ -786,18 +825,17 @@ static int sum_c(lbm_wenoc* h, long long count, double* out) {
     const float* src = classes ? reinterpret_cast<const float*>(h->ws + h->L.ctot) : a.c;
     lw::sum_kernel<float><<<blocks, lw::kReduceThreads, 0, h->stream>>>(a, src, count);
   }
-  if (cudaGetLastError() != cudaSuccess) return LW_ECUDA;
-  if (cudaStreamSynchronize(h->stream) != cudaSuccess) return LW_ECUDA;
-  if (cudaMemcpy(out, h->ws + h->L.scalars + sizeof(double), sizeof(double), cudaMemcpyDeviceToHost) !=
-      cudaSuccess)
-    return LW_ECUDA;
-  return LW_OK;
+  return cudaGetLastError() == cudaSuccess ? LW_OK : LW_ECUDA;
 }
 
 int lbm_wenoc_total_mass(lbm_wenoc* h, double* out) {
   if (!h || !out) return LW_EINVAL;
   if (!h->initialised) return LW_ESTATE;
-  return sum_c(h, h->n, out);
+  int rc = enqueue_sum_c(h, h->n);
+  Readback r;
+  if (rc != LW_OK || (rc = read_back(h, &r)) != LW_OK) return rc;
+  *out = r.scalars[1];
+  return LW_OK;
 }
 
 int lbm_wenoc_mass_below(lbm_wenoc* h, int32_t level, double* out) {
@@ -806,12 +844,13 @@ int lbm_wenoc_mass_below(lbm_wenoc* h, int32_t level, double* out) {
   const int nv = h->p.dim == 3 ? h->p.nz : h->p.ny;
   if (level < 0 || level > nv) return LW_EINVAL;
   // the vertical axis is the slowest: the levels below the plane are the first nodes
-  double below = 0.0, dep = 0.0;
-  int rc = sum_c(h, (long long)level * (h->n / nv), &below);
-  if (rc != LW_OK) return rc;
-  rc = lbm_wenoc_deposited_mass(h, &dep);
+  int rc = fold_late(h);
+  if (rc == LW_OK && level > 0) rc = enqueue_sum_c(h, (long long)level * (h->n / nv));
+  Readback r;
+  if (rc != LW_OK || (rc = read_back(h, &r)) != LW_OK) return rc;
+  rc = status_code(r.status);
   if (rc != LW_OK && rc != LW_EUNSTABLE) return rc;
-  *out = below + dep;
+  *out = (level > 0 ? r.scalars[1] : 0.0) + total_deposit(h, r);
   return rc;
 }
 
@@ -821,9 +860,13 @@ int lbm_wenoc_fields(lbm_wenoc* h, void* rho, void* u, void* c) {
   if (!h->initialised) return LW_ESTATE;
   const size_t es = h->fp64 ? 8 : 4;
   const size_t cbytes = (size_t)h->n * es;
-  // Compute rho and u into the stage buffers (free between steps), then copy out.
-  unsigned char* rho_dev = h->ws + h->L.c2;  // free between steps on every path
-  unsigned char* u_dev = h->ws + h->L.u;
+  // rho and u are computed into the caller's device buffers, or into the stage buffers (free
+  // between steps) and copied out; what is not asked for is not written (except the frozen
+  // velocity's rho)
+  const bool rho_direct = rho && kernel_can_use(h, rho);
+  const bool u_direct = u && !h->frozen && kernel_can_use(h, u);
+  unsigned char* rho_dev = rho_direct ? static_cast<unsigned char*>(rho) : h->ws + h->L.c2;  // free on every path
+  unsigned char* u_dev = u_direct ? static_cast<unsigned char*>(u) : h->ws + h->L.u;
   if (rho || u) {
     if (h->frozen) {
       const int blocks = (int)((h->n + 255) / 256);
@@ -852,8 +895,8 @@ int lbm_wenoc_fields(lbm_wenoc* h, void* rho, void* u, void* c) {
     cudaMemcpyKind k = is_device_pointer(dst) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     return cudaMemcpyAsync(dst, src, nbytes, k, h->stream) == cudaSuccess;
   };
-  if (rho && !copy_out(rho, rho_dev, cbytes)) return LW_ECUDA;
-  if (u && !copy_out(u, u_dev, cbytes * h->p.dim)) return LW_ECUDA;
+  if (rho && !rho_direct && !copy_out(rho, rho_dev, cbytes)) return LW_ECUDA;
+  if (u && !u_direct && !copy_out(u, u_dev, cbytes * h->p.dim)) return LW_ECUDA;
   const size_t c_off = h->ncls > 1 ? h->L.ctot : (h->sweep && h->cur ? h->L.c1 : h->L.c);
   if (c && !copy_out(c, h->ws + c_off, cbytes)) return LW_ECUDA;
   if (cudaStreamSynchronize(h->stream) != cudaSuccess) return LW_ECUDA;
@@ -1021,12 +1064,11 @@ int lbm_wenoc_class(lbm_wenoc* h, int32_t k, void* out) {
 int lbm_wenoc_class_deposit(lbm_wenoc* h, int32_t k, double* out) {
   if (!h || !out || h->ncls < 2 || k < 0 || k >= h->ncls) return LW_EINVAL;
   if (!h->initialised) return LW_ESTATE;
-  int rc = sync_and_status(h);
-  if (rc == LW_ECUDA) return rc;
-  if (cudaMemcpy(out, h->ws + h->L.scalars + sizeof(double) * (kClassDeposit + k), sizeof(double),
-                 cudaMemcpyDeviceToHost) != cudaSuccess)
-    return LW_ECUDA;
-  return rc;
+  Readback r;
+  const int rc = read_back(h, &r);
+  if (rc != LW_OK) return rc;
+  *out = r.scalars[kClassDeposit + k];
+  return status_code(r.status);
 }
 
 int lbm_wenoc_sugar(lbm_wenoc* h, void* S_out) {
