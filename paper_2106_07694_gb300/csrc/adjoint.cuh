@@ -436,6 +436,7 @@ __global__ void __launch_bounds__(128) adj_gather_fluid_kernel(Args<T> a, AdjFie
 template <typename T>
 __global__ void __launch_bounds__(128) adj_fluid_kernel(Args<T> a, AdjFields<T> f, const T* rho_rec, const T* lam_next,
                                                         T* lam_out) {
+  after_previous();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y;
   if (x >= a.nx) return;

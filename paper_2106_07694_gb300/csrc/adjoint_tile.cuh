@@ -119,6 +119,7 @@ __device__ __forceinline__ float column_ed(const AdjTileSmem& S, int half, int j
 // faces, the floor face -Vs c_0 and the deposit's weights) go to this CTA's partial.
 template <int STAGE>
 __global__ void __launch_bounds__(kAT, 4) adj_stage_kernel(Args<float> a, AdjFields<float> f) {
+  after_previous();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   AdjTileSmem& S = *reinterpret_cast<AdjTileSmem*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -369,7 +370,7 @@ inline cudaError_t adj_stage_prepare() {
 template <int STAGE>
 inline void launch_adj_stage(const Args<float>& a, const AdjFields<float>& f, cudaStream_t s) {
   const dim3 grid((a.nx + kAx - 1) / kAx, (a.ny + kAy - 1) / kAy);
-  adj_stage_kernel<STAGE><<<grid, kAT, sizeof(AdjTileSmem), s>>>(a, f);
+  launch_dependent(adj_stage_kernel<STAGE>, grid, kAT, sizeof(AdjTileSmem), s, a, f);
 }
 
 }  // namespace lw

@@ -43,10 +43,12 @@ struct Args {
   int late_count;  // deposit folded late (fold_late_deposit): partials a step's last stage leaves; 0 = it folds them
 };
 
-// Global-load policies.  LoadNC reads through the non-coherent (read-only) path, for data
-// no thread writes while the kernel runs; LoadL2 reads at L2 (ld.global.cg: no L1 line is
+// Global-load policies.  LoadPlain is an ordinary load, for a kernel that may have been started
+// before the one ahead of it ended (launch_dependent): it reads what that one wrote, so the
+// read-only path is closed to it.  LoadNC reads through the non-coherent (read-only) path, for
+// data no thread writes while the kernel runs.  LoadL2 reads at L2 (ld.global.cg: no L1 line is
 // kept), for a kernel that reads what other CTAs wrote earlier in the same launch, after
-// a grid barrier; LoadPlain is an ordinary load.
+// a grid barrier.
 struct LoadNC {
   static __device__ __forceinline__ float s(const float* p) { return __ldg(p); }
   static __device__ __forceinline__ double s(const double* p) { return __ldg(p); }
@@ -91,6 +93,29 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+
+// Programmatic dependent launch: a kernel launched by launch_dependent() has its launch and
+// its CTAs' start processed while the one before it on the stream drains; after_previous(),
+// its first statement, waits until that one has ended and its writes are visible, so no
+// global memory is touched early.  Nothing triggers the next launch before a CTA's end: with
+// the trigger at a kernel's start the next grids' waiting CTAs took the slots unevenly (the
+// 128 x 256 FP64 step went from 97 to 259 us); without it a launch costs about 0.25 us less.
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                    const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
 
 // fused multiply-add of the kernel's precision (fmaf for FP32, fma for FP64)
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }

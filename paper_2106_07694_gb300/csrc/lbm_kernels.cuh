@@ -154,12 +154,14 @@ __device__ __forceinline__ void lbm_d2q9_body(const Args<T>& a, int bx, int by, 
 
 template <typename T, int PARITY, bool SUGAR = false>
 __global__ void __launch_bounds__(128) lbm_d2q9_kernel(Args<T> a) {
+  after_previous();
   lbm_d2q9_body<T, PARITY, false, SUGAR>(a, blockIdx.x, blockIdx.y);
 }
 
 // The same step that also stores rho (the steps recorded for the adjoint).
 template <typename T, int PARITY>
 __global__ void __launch_bounds__(128) lbm_d2q9_record_kernel(Args<T> a, T* rho_out) {
+  after_previous();
   lbm_d2q9_body<T, PARITY, true>(a, blockIdx.x, blockIdx.y, rho_out);
 }
 
@@ -196,7 +198,7 @@ __device__ __forceinline__ D2Q9Node d2q9_node(const Args<T>& a, int x, int y) {
 }
 
 // The node's populations as they stand at the start of a step of this parity (AA pattern).
-template <typename T, int PARITY, class LD = LoadNC>
+template <typename T, int PARITY, class LD = LoadPlain>
 __device__ __forceinline__ void d2q9_load(const Args<T>& a, const D2Q9Node& nd, T (&g)[9]) {
   const unsigned n = (unsigned)a.n;
   const T* __restrict__ G = a.g;

@@ -295,7 +295,7 @@ void enqueue_sugar(lbm_wenoc* h, const Args<T>& a) {
   const dim3 blk(lw::kSugarX, lw::kSugarY);
   const dim3 grd(lw::sugar_blocks_x(a.nx) * (unsigned)(((long long)a.ny * a.nz + lw::kSugarY - 1) / lw::kSugarY));
   cudaStream_t s = h->stream;
-  launch(h, K_SUGAR, [&] { lw::sugar_kernel<T, LAT::DIM><<<grd, blk, 0, s>>>(a); });
+  launch(h, K_SUGAR, [&] { lw::launch_dependent(lw::sugar_kernel<T, LAT::DIM>, grd, blk, 0, s, a); });
   h->cur ^= 1;
 }
 
@@ -316,7 +316,7 @@ void enqueue_class_sum(lbm_wenoc* h) {
   const long long quads = h->n / 4;
   T* out = reinterpret_cast<T*>(h->ws + h->L.ctot);
   launch(h, K_OTHER, [&] {
-    lw::class_sum_kernel<T><<<(unsigned)((quads + 255) / 256), 256, 0, h->stream>>>(cp, out, quads);
+    lw::launch_dependent(lw::class_sum_kernel<T>, (unsigned)((quads + 255) / 256), 256, 0, h->stream, cp, out, quads);
   });
 }
 
@@ -332,12 +332,12 @@ void enqueue_step(lbm_wenoc* h, int parity) {
     launch(h, K_LBM, [&] {
       if (LAT::DIM == 2) {
         if (h->sugar)
-          parity == 0 ? lw::lbm_d2q9_kernel<T, 0, true><<<grd, blk, 0, s>>>(af)
-                      : lw::lbm_d2q9_kernel<T, 1, true><<<grd, blk, 0, s>>>(af);
+          parity == 0 ? lw::launch_dependent(lw::lbm_d2q9_kernel<T, 0, true>, grd, blk, 0, s, af)
+                      : lw::launch_dependent(lw::lbm_d2q9_kernel<T, 1, true>, grd, blk, 0, s, af);
         else if (parity == 0)
-          lw::lbm_d2q9_kernel<T, 0><<<grd, blk, 0, s>>>(af);
+          lw::launch_dependent(lw::lbm_d2q9_kernel<T, 0>, grd, blk, 0, s, af);
         else
-          lw::lbm_d2q9_kernel<T, 1><<<grd, blk, 0, s>>>(af);
+          lw::launch_dependent(lw::lbm_d2q9_kernel<T, 1>, grd, blk, 0, s, af);
       } else {
         if (h->sugar)
           parity == 0 ? lw::lbm_d3q19_kernel<T, 0, true><<<grd, blk, 0, s>>>(af)
@@ -1656,9 +1656,9 @@ int record_step(lbm_wenoc* h, const StepRecord<T>& R, bool first, T* next) {
   const dim3 blk(kLbmThreads), grd((a.nx + kLbmThreads - 1) / kLbmThreads, a.ny, 1);
   launch(h, K_LBM, [&] {
     if (h->parity == 0)
-      lw::lbm_d2q9_record_kernel<T, 0><<<grd, blk, 0, s>>>(a, R.rho);
+      lw::launch_dependent(lw::lbm_d2q9_record_kernel<T, 0>, grd, blk, 0, s, a, R.rho);
     else
-      lw::lbm_d2q9_record_kernel<T, 1><<<grd, blk, 0, s>>>(a, R.rho);
+      lw::launch_dependent(lw::lbm_d2q9_record_kernel<T, 1>, grd, blk, 0, s, a, R.rho);
   });
   enqueue_transport<D2Q9, T>(h, a, h->stage2d && next ? next : c_own);
   h->parity ^= 1;
@@ -1682,7 +1682,7 @@ int adjoint_step(lbm_wenoc* h, const StepRecord<T>& R, const lw::AdjFields<T>& f
     launch(h, K_ADJ_FACES, [&] { lw::launch_adj_stage<3>(a, f, s); });
     launch(h, K_ADJ_FACES, [&] { lw::launch_adj_stage<2>(a, f, s); });
     launch(h, K_ADJ_FACES, [&] { lw::launch_adj_stage<1>(a, f, s); });
-    launch(h, K_ADJ_FLUID, [&] { lw::adj_fluid_kernel<T><<<grd, blk, 0, s>>>(a, f, R.rho, lam_next, lam_out); });
+    launch(h, K_ADJ_FLUID, [&] { lw::launch_dependent(lw::adj_fluid_kernel<T>, grd, blk, 0, s, a, f, R.rho, lam_next, lam_out); });
   } else {
     launch(h, K_ADJ_FACES, [&] { lw::adj_faces_kernel<T, 3><<<grd, blk, 0, s>>>(a, f, fr); });
     launch(h, K_ADJ_GATHER, [&] { lw::adj_gather_kernel<T, 3><<<grd, blk, 0, s>>>(a, f, fr); });

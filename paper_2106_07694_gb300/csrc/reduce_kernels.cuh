@@ -92,6 +92,7 @@ struct ClassPtrs {
 // the sum runs in class order, four nodes per thread.
 template <typename T>
 __global__ void class_sum_kernel(ClassPtrs<T> cp, T* out, long long quads) {
+  after_previous();
   const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (k >= quads) return;
   Quad<T> v[8];

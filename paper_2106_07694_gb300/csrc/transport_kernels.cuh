@@ -207,6 +207,7 @@ __host__ __device__ __forceinline__ unsigned sugar_blocks_x(int nx) { return (un
 
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kSugarX * kSugarY) sugar_kernel(Args<T> a) {
+  after_previous();
   const int nx = a.nx, ny = a.ny, nz = a.nz;
   const unsigned gx = sugar_blocks_x(nx);  // blocks along x; every block in grid.x, which has no 65535 limit
   const int x = 4 * (int)(blockIdx.x % gx * kSugarX + threadIdx.x);

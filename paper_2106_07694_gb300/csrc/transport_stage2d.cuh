@@ -69,11 +69,11 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
   auto fetch_row = [&](int k) {
     if (k >= y1) return;
     const unsigned row = (unsigned)k * (unsigned)nx;
-    p0c = __ldg(cin + row + gxs);
-    p0u = __ldg(ux + row + gxs);
+    p0c = LoadPlain::s(cin + row + gxs);
+    p0u = LoadPlain::s(ux + row + gxs);
     if (has2) {
-      p1c = __ldg(cin + row + gx1);
-      p1u = __ldg(ux + row + gx1);
+      p1c = LoadPlain::s(cin + row + gx1);
+      p1u = LoadPlain::s(ux + row + gx1);
     }
   };
   // own column, row l (ghost rows reflect): value and scaled vertical velocity
@@ -82,10 +82,10 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
     const bool ghost = l < 0 || l >= ny;
     const int lr = l < 0 ? -1 - l : (l >= ny ? 2 * ny - 1 - l : l);
     const unsigned k = (unsigned)lr * (unsigned)nx + X;
-    qc = __ldg(cin + k);
-    const T u = __ldg(uy + k);
+    qc = LoadPlain::s(cin + k);
+    const T u = LoadPlain::s(uy + k);
     // with sugar the settling velocity of the node (a ghost reads its mirror's) is Vs (1 - ks S)
-    const T vsa = SUGAR ? vs_a * fma_t(-a.ks, __ldg(a.S + k), T(1)) : vs_a;
+    const T vsa = SUGAR ? vs_a * fma_t(-a.ks, LoadPlain::s(a.S + k), T(1)) : vs_a;
     qw = fma_t(ghost ? -u : u, inv_alpha, -vsa);
   };
   constexpr bool SIGN = (SCHEME & kSchemeSignSplit) != 0;
@@ -185,7 +185,7 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
 
     // ---- divergence and the Shu-Osher combination of this stage
     if (!prime) {
-      const T vs_floor = SUGAR && k == 0 ? a.vs * fma_t(-a.ks, __ldg(a.S + X), T(1)) : a.vs;
+      const T vs_floor = SUGAR && k == 0 ? a.vs * fma_t(-a.ks, LoadPlain::s(a.S + X), T(1)) : a.vs;
       const T Lk = S.fx[t] - S.fx[t + 1] + (carry - fup);  // carry is 0 below the floor row
       const T cb = k == 0 ? fma_t(-vs_floor, chere, chere) : chere;  // less the floor outflow
       if (out) {
@@ -235,6 +235,7 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
 
 template <int STAGE, bool SUGAR = false, int SCHEME = 0, typename T = float>
 __global__ void __launch_bounds__(kS2T) rk_stage2d_kernel(Args<T> a, Stage2dParamsT<T> sp) {
+  after_previous();
   stage2d_body<STAGE, SUGAR, SCHEME, T>(a, sp, blockIdx.x, blockIdx.y, gridDim.x);
 }
 
@@ -255,16 +256,16 @@ template <int STAGE, bool SUGAR, typename T>
 inline void launch_stage2d_scheme(const Args<T>& a, const Stage2dParamsT<T>& sp, dim3 grid, cudaStream_t s) {
   switch (a.scheme) {
     case kSchemeWeno3:
-      rk_stage2d_kernel<STAGE, SUGAR, kSchemeWeno3, T><<<grid, kS2T, 0, s>>>(a, sp);
+      launch_dependent(rk_stage2d_kernel<STAGE, SUGAR, kSchemeWeno3, T>, grid, kS2T, 0, s, a, sp);
       break;
     case kSchemeSignSplit:
-      rk_stage2d_kernel<STAGE, SUGAR, kSchemeSignSplit, T><<<grid, kS2T, 0, s>>>(a, sp);
+      launch_dependent(rk_stage2d_kernel<STAGE, SUGAR, kSchemeSignSplit, T>, grid, kS2T, 0, s, a, sp);
       break;
     case kSchemeWeno3 | kSchemeSignSplit:
-      rk_stage2d_kernel<STAGE, SUGAR, kSchemeWeno3 | kSchemeSignSplit, T><<<grid, kS2T, 0, s>>>(a, sp);
+      launch_dependent(rk_stage2d_kernel<STAGE, SUGAR, kSchemeWeno3 | kSchemeSignSplit, T>, grid, kS2T, 0, s, a, sp);
       break;
     default:
-      rk_stage2d_kernel<STAGE, SUGAR, 0, T><<<grid, kS2T, 0, s>>>(a, sp);
+      launch_dependent(rk_stage2d_kernel<STAGE, SUGAR, 0, T>, grid, kS2T, 0, s, a, sp);
   }
 }
 

@@ -154,9 +154,9 @@ __device__ __forceinline__ float4 column_faces(const float4 (&P)[6], const float
 }
 
 // SUGAR: the settling velocity of a node is Vs (1 - ks S).  SCHEME: transport-scheme variant
-// bits (face_flux_scheme).  LD: the global-load policy (LoadNC for a launch of its own, LoadL2
+// bits (face_flux_scheme).  LD: the global-load policy (LoadPlain for a launch of its own, LoadL2
 // inside a kernel whose earlier phases wrote the fields).
-template <int STAGE, bool SUGAR = false, int SCHEME = 0, class LD = LoadNC>
+template <int STAGE, bool SUGAR = false, int SCHEME = 0, class LD = LoadPlain>
 __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<float>& a, const Stage2dParams& sp,
                                                   int bx, int by, int strips) {
   const int t = threadIdx.x;
@@ -417,6 +417,7 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
 
 template <int STAGE, bool SUGAR = false, int SCHEME = 0>
 __global__ void __launch_bounds__(kWT, kWminB) rk_stage2d_wide_kernel(Args<float> a, Stage2dParams sp) {
+  after_previous();
   __shared__ __align__(16) StageWideSmem S;
   stage2d_wide_body<STAGE, SUGAR, SCHEME>(S, a, sp, blockIdx.x, blockIdx.y, gridDim.x);
 }
@@ -470,7 +471,7 @@ inline cudaError_t launch_stage2d_wide(const Args<float>& a, const float* cin, f
   sp.cout = cout;
   sp.H = H;
   const dim3 grid((a.nx + kWW - 1) / kWW, (a.ny + H - 1) / H);
-  stage2d_wide_entry<STAGE>(a.S != nullptr, a.scheme)<<<grid, kWT, 0, s>>>(a, sp);
+  launch_dependent(stage2d_wide_entry<STAGE>(a.S != nullptr, a.scheme), grid, kWT, 0, s, a, sp);
   return cudaGetLastError();
 }
 

@@ -49,6 +49,7 @@ struct Tile2dSmem {
 
 template <int STAGE, bool SUGAR = false, int SCHEME = 0>
 __global__ void __launch_bounds__(kTT, 1024 / kTT) rk_tile2d_kernel(Args<float> a, Stage2dParams sp) {
+  after_previous();
   constexpr int TX = kTX, TY = kTY, T = kTT;
   __shared__ __align__(16) Tile2dSmem S;
   const int tid = threadIdx.x;
@@ -81,11 +82,11 @@ __global__ void __launch_bounds__(kTT, 1024 / kTT) rk_tile2d_kernel(Args<float> 
       gx = gx < 0 ? gx + nx : gx;
       while (gx >= nx) gx -= nx;
       const unsigned node = (unsigned)lr * (unsigned)nx + (unsigned)gx;
-      const float4 c = LoadNC::v4(cin + node);
+      const float4 c = LoadPlain::v4(cin + node);
       float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u, s = u;
-      if (in_row) u = LoadNC::v4(ux + node);
-      if (in_col) v = LoadNC::v4(uy + node);
-      if (SUGAR && in_col) s = LoadNC::v4(a.S + node);
+      if (in_row) u = LoadPlain::v4(ux + node);
+      if (in_col) v = LoadPlain::v4(uy + node);
+      if (SUGAR && in_col) s = LoadPlain::v4(a.S + node);
       *reinterpret_cast<float4*>(&S.c[r][4 * q]) = c;
       float4 P, M;
       if (in_row) {
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__(kTT, 1024 / kTT) rk_tile2d_kernel(Args<float> 
   const bool out = y < ny && xl < nx;
   const unsigned node = (unsigned)y * (unsigned)nx + (unsigned)xl;
   float4 cn = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (STAGE > 1 && out) cn = LoadNC::v4(a.c + node);
+  if (STAGE > 1 && out) cn = LoadPlain::v4(a.c + node);
   float fxq[4], fr;
   float4 cq;
   {
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(kTT, 1024 / kTT) rk_tile2d_kernel(Args<float> 
     float vsf[4] = {a.vs, a.vs, a.vs, a.vs};
     if (y == 0) {  // the floor row's settling outflow
       if (SUGAR) {
-        const float4 s0 = LoadNC::v4(a.S + xl);
+        const float4 s0 = LoadPlain::v4(a.S + xl);
         vsf[0] *= fmaf(-a.ks, s0.x, 1.f);
         vsf[1] *= fmaf(-a.ks, s0.y, 1.f);
         vsf[2] *= fmaf(-a.ks, s0.z, 1.f);
@@ -205,7 +206,7 @@ __global__ void __launch_bounds__(kTT, 1024 / kTT) rk_tile2d_kernel(Args<float> 
     if (STAGE == 3) {
       report_status(a.status, !(isfinite(v[0]) && isfinite(v[1]) && isfinite(v[2]) && isfinite(v[3])));
       if (y == 0) {  // RK3 b-weights of the floor flux: c^n/6 + c1/6 + 2 c2/3
-        const float4 c1 = LoadNC::v4(a.c1 + xl);
+        const float4 c1 = LoadPlain::v4(a.c1 + xl);
         const float c1v[4] = {c1.x, c1.y, c1.z, c1.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -270,7 +271,7 @@ inline cudaError_t launch_tile2d(const Args<float>& a, const float* cin, float* 
   sp.cout = cout;
   sp.H = kTY;
   const dim3 grid((a.nx + kTX - 1) / kTX, (a.ny + kTY - 1) / kTY + (STAGE == 1 && a.late_count > 0 ? 1 : 0));
-  tile2d_entry<STAGE>(a.S != nullptr, a.scheme)<<<grid, kTT, 0, s>>>(a, sp);
+  launch_dependent(tile2d_entry<STAGE>(a.S != nullptr, a.scheme), grid, kTT, 0, s, a, sp);
   return cudaGetLastError();
 }
 
