@@ -1191,6 +1191,20 @@ void batch_destroy_graphs(lbm_wenoc_batch* b) {
   }
 }
 
+// Rows per segment of the stage items unless the autotuner chose others, one height for the
+// whole batch.  With N nodes over `grid` CTAs that take items as they come, an item of H rows
+// costs about H + 2 (ring fill, priming row) and the last ones end H + 2 rows apart, half of
+// that on average: N / (256 grid) (1 + 2/H) + (H + 2)/2 rows, least at H = 2 sqrt(N / (256 grid)).
+// 64 instances, 56 M nodes: 27; a step takes 2.52 ms with each instance's own height for a run
+// alone (2 to 20 rows, sized to fill the chip by itself), 2.23 ms at 32 rows, 2.25 at 48, 2.29
+// at 64.
+int batch_default_rows(const lbm_wenoc_batch* b) {
+  double nodes = 0.0;
+  for (const lbm_wenoc* h : b->inst) nodes += (double)h->n;
+  const double per = nodes / ((double)lw::kWW * std::max(1, b->grid));
+  return std::max(2, std::min(lw::kWmaxH, (int)std::lround(2.0 * std::sqrt(per))));
+}
+
 // Fill the device tables from the instances' current argument blocks and geometries.
 int batch_upload_tables(lbm_wenoc_batch* b) {
   const int count = (int)b->inst.size();
@@ -1198,6 +1212,7 @@ int batch_upload_tables(lbm_wenoc_batch* b) {
   std::vector<int> lstart(count + 1), lgx(count), sstart(count + 1), sstrips(count), srows(count), fstart(count + 1),
       fchunks(count);
   lstart[0] = sstart[0] = fstart[0] = 0;
+  const int batch_rows = batch_default_rows(b);
   for (int i = 0; i < count; ++i) {
     lbm_wenoc* h = b->inst[i];
     args[i] = make_args<float>(h);
@@ -1205,7 +1220,7 @@ int batch_upload_tables(lbm_wenoc_batch* b) {
     lgx[i] = (h->p.nx + kLbmThreads - 1) / kLbmThreads;
     lstart[i + 1] = lstart[i] + lgx[i] * h->p.ny;
     sstrips[i] = (h->p.nx + lw::kWW - 1) / lw::kWW;
-    srows[i] = std::min(std::min(b->rows[i] > 0 ? b->rows[i] : h->stage2d_rows, h->p.ny), lw::kWmaxH);
+    srows[i] = std::min(std::min(b->rows[i] > 0 ? b->rows[i] : batch_rows, h->p.ny), lw::kWmaxH);
     const int segs = (h->p.ny + srows[i] - 1) / srows[i];
     sstart[i + 1] = sstart[i] + sstrips[i] * segs;
     fchunks[i] = (h->p.nx + lw::kFluidCols - 1) / lw::kFluidCols;
@@ -1500,10 +1515,11 @@ int lbm_wenoc_batch_autotune(lbm_wenoc_batch* b, int32_t steps_per_trial, int32_
   if (rc != LW_OK) return rc;
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return LW_ECUDA;
-  // start from each instance's own heuristic, then one pass of coordinate descent over the
+  // start from the batch's default height, then one pass of coordinate descent over the
   // shape classes (instances of one lattice size share a segment height): try each
   // candidate height for the class with the whole batch timed, keep the fastest
-  for (int i = 0; i < count; ++i) b->rows[i] = b->inst[i]->stage2d_rows;
+  for (int i = 0; i < count; ++i)
+    b->rows[i] = std::min(batch_default_rows(b), std::min(b->inst[i]->p.ny, lw::kWmaxH));
   std::vector<std::pair<int, int>> shapes;
   for (lbm_wenoc* h : b->inst) {
     const std::pair<int, int> sh(h->p.nx, h->p.ny);
