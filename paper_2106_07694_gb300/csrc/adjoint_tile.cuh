@@ -135,23 +135,39 @@ __global__ void __launch_bounds__(kAT, 4) adj_stage_kernel(Args<float> a, AdjFie
 
   // ---- stage the tile and its halo cross
   constexpr int kQ = kAx / 4 + 2, kPos = (kAy + 8) * kQ;
-  for (int p = tid; p < kPos; p += kAT) {
-    const int row = p / kQ, q = p % kQ;
+  constexpr int kRounds = (kPos + kAT - 1) / kAT;
+  Quad<float> Lc[kRounds], Ll[kRounds], Lx[kRounds], Ly[kRounds];
+#pragma unroll
+  for (int k = 0; k < kRounds; ++k) {  // all loads in flight together
+    const int p = tid + k * kAT, row = p / kQ, q = p % kQ;
     const bool in_row = row >= 4 && row < kAy + 4, in_col = q >= 1 && q <= kAx / 4;
-    if (!in_row && !in_col) continue;
+    if (p >= kPos || (!in_row && !in_col)) continue;
     const int gr = y0 - 4 + row;
-    const bool ghost = gr < 0 || gr >= ny;
     int lr = gr < 0 ? -1 - gr : (gr >= ny ? 2 * ny - 1 - gr : gr);
     lr = max(0, min(ny - 1, lr));  // rows past the ghosts that a face reads: any value
-    const int gx = ((x0 - 4 + 4 * q) % nx + nx) % nx;
+    int gx = x0 - 4 + 4 * q;
+    gx = gx < 0 ? gx + nx : gx;
+    while (gx >= nx) gx -= nx;
     const unsigned node = (unsigned)lr * (unsigned)nx + (unsigned)gx;
-    const Quad<float> c = load_quad(cs + node), l = load_quad(lsrc + node);
+    Lc[k] = load_quad(cs + node);
+    Ll[k] = load_quad(lsrc + node);
+    if (in_row) Lx[k] = load_quad(ux + node);
+    if (in_col) Ly[k] = load_quad(uy + node);
+  }
+#pragma unroll
+  for (int k = 0; k < kRounds; ++k) {
+    const int p = tid + k * kAT, row = p / kQ, q = p % kQ;
+    const bool in_row = row >= 4 && row < kAy + 4, in_col = q >= 1 && q <= kAx / 4;
+    if (p >= kPos || (!in_row && !in_col)) continue;
+    const int gr = y0 - 4 + row;
+    const bool ghost = gr < 0 || gr >= ny;
+    const Quad<float> c = Lc[k];
     Quad<float> P, M;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) P.v[j] = lscale * l.v[j];
+    for (int j = 0; j < 4; ++j) P.v[j] = lscale * Ll[k].v[j];
     *reinterpret_cast<Quad<float>*>(&S.lam[row][4 * q]) = P;
     if (in_row) {
-      const Quad<float> u = load_quad(ux + node);
+      const Quad<float> u = Lx[k];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const float h = 0.5f * c.v[j], w = u.v[j] * ia;
@@ -162,7 +178,7 @@ __global__ void __launch_bounds__(kAT, 4) adj_stage_kernel(Args<float> a, AdjFie
       *reinterpret_cast<Quad<float>*>(&S.mx[row - 4][4 * q]) = M;
     }
     if (in_col) {
-      const Quad<float> u = load_quad(uy + node);
+      const Quad<float> u = Ly[k];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const float h = 0.5f * c.v[j], w = ((ghost ? -u.v[j] : u.v[j]) - vs) * ia;
@@ -211,13 +227,21 @@ __global__ void __launch_bounds__(kAT, 4) adj_stage_kernel(Args<float> a, AdjFie
   y_block(I0(), I4(), warp, lane);
   if (warp == 0) y_block(I2(), I4(), -1, lane);
   if (warp == 1) y_block(I0(), I3(), kAy / 4, lane);
+  // c and u_y of this thread's four rows, on their way during the barrier
+  float yc[4], yu[4];
+  const int ycol = x0 + lane < nx ? x0 + lane : (x0 + lane) % nx;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const unsigned node = (unsigned)min(y0 + 4 * warp + j, ny - 1) * (unsigned)nx + (unsigned)ycol;
+    yc[j] = cs[node];
+    yu[j] = uy[node];
+  }
   __syncthreads();
 
   // ---- y part of the tile's nodes: four rows of one column
   float vs_acc = 0.f;
   {
     const int col = lane, r0 = 4 * warp;
-    const int X = (x0 + col) % nx;
     const bool own = x0 + col < nx;
     float lamF[5], edP[5], edM[5];
 #pragma unroll
@@ -231,8 +255,7 @@ __global__ void __launch_bounds__(kAT, 4) adj_stage_kernel(Args<float> a, AdjFie
       const int r = r0 + j, y = y0 + r;
       float gc = 0.f, gw = 0.f;
       if (y < ny) {
-        const unsigned node = (unsigned)y * (unsigned)nx + (unsigned)X;
-        const float c = cs[node], u = uy[node];
+        const float c = yc[j], u = yu[j];
         const float GP = edP[j] - edP[j + 1] + lamF[j + 1], GM = edM[j] - edM[j + 1] + lamF[j];
         const float wa = (u - vs) * ia, hc = 0.5f * c;
         gc = fmaf(0.5f * alpha, fmaf(GP, wa + 1.f, GM * (wa - 1.f)), kappa * (lamF[j + 1] - lamF[j]));
@@ -286,14 +309,28 @@ __global__ void __launch_bounds__(kAT, 4) adj_stage_kernel(Args<float> a, AdjFie
   x_block(I0(), I4(), q, row);
   if (warp == 2) x_block(I2(), I4(), -1, lane);
   if (warp == 3) x_block(I0(), I3(), kAx / 4, lane);
+  // the fields of this thread's four nodes, on their way during the barrier
+  const int y = y0 + row, xl = x0 + 4 * q;
+  const bool own = y < ny && xl < nx;
+  const unsigned node = (unsigned)y * (unsigned)nx + (unsigned)xl;
+  Quad<float> c{}, u{}, mu{}, l2{}, ox{}, oy{};
+  if (own) {
+    c = load_quad(cs + node);
+    u = load_quad(ux + node);
+    if (STAGE == 1) {
+      mu = load_quad(f.mu + node);
+      l2 = load_quad(f.lc2 + node);
+    }
+    if (STAGE < 3) {
+      ox = load_quad(f.lam_u + node);
+      oy = load_quad(f.lam_u + n + node);
+    }
+  }
   __syncthreads();
 
   // ---- the tile's nodes: four columns of one row
   {
-    const int y = y0 + row, xl = x0 + 4 * q;
-    if (y < ny && xl < nx) {
-      const unsigned node = (unsigned)y * (unsigned)nx + (unsigned)xl;
-      const Quad<float> c = load_quad(cs + node), u = load_quad(ux + node);
+    if (own) {
       auto sum4 = [](const float4& p, const float4& r) { return make_float4(p.x + r.x, p.y + r.y, p.z + r.z, p.w + r.w); };
       float edP[5], edM[5], lamF[5];
       {
@@ -328,12 +365,10 @@ __global__ void __launch_bounds__(kAT, 4) adj_stage_kernel(Args<float> a, AdjFie
         gy.v[j] = S.my[row][4 * q + j];
       }
       if (STAGE == 1) {
-        const Quad<float> mu = load_quad(f.mu + node), l2 = load_quad(f.lc2 + node);
 #pragma unroll
         for (int j = 0; j < 4; ++j) v.v[j] += fmaf(1.f / 3.f, mu.v[j], 0.75f * l2.v[j]);
       }
       if (STAGE < 3) {
-        const Quad<float> ox = load_quad(f.lam_u + node), oy = load_quad(f.lam_u + n + node);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           gx.v[j] += ox.v[j];
