@@ -182,7 +182,8 @@ int64_t lbm_wenoc_launch_count(const lbm_wenoc* h);
 
 /* Tuning of the FP32 transport sweeps: rows per CTA segment of the 2D stage kernels (or
  * of the fused 2D kernel), or z levels per CTA segment of the 3D stage kernels (0 = default).  Results do not
- * depend on it (bitwise).  No effect on FP64 or periodic-vertical handles.  Drops
+ * depend on it (bitwise).  No effect on 3D FP64 or periodic-vertical handles, nor on the 2D FP32
+ * lattices small enough to run on tiles (3.5 M nodes).  Drops
  * captured graphs; call between steps. */
 int lbm_wenoc_set_segment_rows(lbm_wenoc* h, int32_t rows);
 

@@ -146,7 +146,7 @@ struct lbm_wenoc {
   bool wide = false;     // ... with four columns per thread (FP32, without LW_ONE_COLUMN)
   bool tile = false;     // ... on tiles (four-column handles whose lattice stays in L2)
   int late_count = 0;    // partials of the deposit folded late (0: the last stage folds them)
-  bool late_pending = false;  // a step since the last fold
+  bool late_pending = false;  // a step of this handle since the last fold
   int wide_per_sm = 1;   // CTAs of the four-column stage kernel one SM holds at once
   bool initialised = false;
   bool sugar = false;  // LW_SUGAR: S in L.sa / L.sb, selected by cur (the generic transport path)
@@ -550,9 +550,11 @@ bool kernel_can_use(const lbm_wenoc* h, const void* p) {
          reinterpret_cast<uintptr_t>(p) % (h->fp64 ? 8u : 4u) == 0;
 }
 
-// Fold the deposit of the last step where that was left to the next one.
+// Fold the deposit of the last step where that was left to the next one.  Not only when this
+// handle knows of a step since the last fold: steps that a caller captured into a graph of its own
+// are replayed without it.  With nothing left the partials are zero.
 int fold_late(lbm_wenoc* h) {
-  if (!h->late_pending) return LW_OK;
+  if (h->late_count == 0) return LW_OK;
   h->late_pending = false;
   const Args<float> a = make_args<float>(h);  // FP32 handles only
   lw::late_deposit_kernel<float><<<1, 32, 0, h->stream>>>(a);
@@ -1338,7 +1340,8 @@ int batch_advance(lbm_wenoc_batch* b, int64_t nsteps, bool require_init) {
   for (lbm_wenoc* h : b->inst) {
     if (require_init && !h->initialised) return LW_ESTATE;
     if (h->parity != par || h->steps != b->inst[0]->steps) return LW_ESTATE;
-    if (int rc = fold_late(h)) return rc;  // of an instance stepped alone before
+    if (h->late_pending)  // an instance stepped alone before
+      if (int rc = fold_late(h)) return rc;
   }
   int64_t left = nsteps;
   int parity = par;

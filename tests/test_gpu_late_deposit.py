@@ -52,6 +52,28 @@ def test_deposit_does_not_depend_on_when_it_is_read(shape, extra):
             assert np.array_equal(to_np(a), to_np(b))
 
 
+def test_steps_replayed_from_a_callers_graph():
+    # an even number of steps (the population layout is back where it was), replayed twice
+    from paper_2106_07694_gb300.lbm_wenoc import Simulation
+    shape = (100, 33)
+    c0 = workloads.interface_field(shape, interface_frac=0.3, amplitude=0.03, seed=43, lower=0.2)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        s, ref = (Simulation(shape, graphs=False, **KW) for _ in range(2))
+        for k in (s, ref):
+            k.init(torch.from_numpy(c0.astype(np.float32)).cuda())
+        stream.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            s.step(2)
+        for n in range(3):
+            g.replay()
+            ref.step(2)
+            assert s.deposit == ref.deposit
+        for a, b in zip(s.fields(), ref.fields()):
+            assert np.array_equal(to_np(a), to_np(b))
+
+
 def test_instances_stepped_alone_then_together():
     from paper_2106_07694_gb300 import lbm_wenoc as lw
     from paper_2106_07694_gb300.lbm_wenoc import Batch, Simulation
