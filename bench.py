@@ -162,29 +162,28 @@ class ClockSampler:
 
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from the ncu
-# launch lists summarised in profiles/ (the bench command itself, one pass per launch), with
-# the SHA-1 prefix of the kernel sources they were taken on (the kernel's file and the
-# headers it includes, concatenated in this order); a changed kernel reports null until it
-# is captured again.  The fluid entry is the mean of the two AA parities.
+# launch lists summarised in profiles/ (the workload run for a few steps, one pass per
+# launch), with the SHA-1 prefix of the kernel sources they were taken on (the kernel's file
+# and the headers it includes, concatenated in this order); a changed kernel reports null
+# until it is captured again.  The fluid entry is the mean of the two AA parities.
 _CSRC = "paper_2106_07694_gb300/csrc/"
 _LBM_SRC = ("lbm_kernels.cuh", "lattice.cuh", "common.cuh")
-_STAGE_SRC = ("transport_stage2d_wide.cuh", "transport_stage2d.cuh", "transport_sweep2d.cuh", "reduce_kernels.cuh",
-              "common.cuh")
+_STAGE_SRC = ("transport_stage2d_wide.cuh", "transport_stage2d.cuh", "weno.cuh", "common.cuh")
 _STAGE3D_SRC = ("transport_sweep3d_wide.cuh", "transport_sweep3d.cuh") + _STAGE_SRC
 NCU_TRAFFIC = {
-    "lbm_collide_stream": (643.1e6, _LBM_SRC, "2097009c2aa4"),
-    "rk_stage1": (134.3e6, _STAGE_SRC, "dd1ee704fac2"),
-    "rk_stage2": (178.4e6, _STAGE_SRC, "dd1ee704fac2"),
-    "rk_stage3": (171.9e6, _STAGE_SRC, "dd1ee704fac2"),
-    # 512 x 1024 adjoint workload (the face records stay in L2)
-    "adj_faces": (8.57e6, ("adjoint.cuh",) + _LBM_SRC, "d60661f5666e"),
+    "lbm_collide_stream": (642.9e6, _LBM_SRC, "7bf409f75720"),
+    "rk_stage1": (131.9e6, _STAGE_SRC, "de250e1536b5"),
+    "rk_stage2": (172.7e6, _STAGE_SRC, "de250e1536b5"),
+    "rk_stage3": (166.2e6, _STAGE_SRC, "de250e1536b5"),
+    # 512 x 1024 adjoint workload, mean of the three stages (step records read from HBM)
+    "adj_faces": (12.65e6, ("adjoint_tile.cuh", "weno.cuh", "adjoint.cuh") + _LBM_SRC, "f046134ff56d"),
 }
 # the 256 x 256 x 512 D3Q19 workload
 NCU_TRAFFIC_3D = {
-    "lbm_collide_stream": (5577.75e6, _LBM_SRC, "2097009c2aa4"),
-    "rk_stage1": (966.4e6, _STAGE3D_SRC, "5a04479acddc"),
-    "rk_stage2": (1127.2e6, _STAGE3D_SRC, "5a04479acddc"),
-    "rk_stage3": (1109.2e6, _STAGE3D_SRC, "5a04479acddc"),
+    "lbm_collide_stream": (5577.7e6, _LBM_SRC, "7bf409f75720"),
+    "rk_stage1": (735.8e6, _STAGE3D_SRC, "520ea50d8f39"),
+    "rk_stage2": (874.6e6, _STAGE3D_SRC, "520ea50d8f39"),
+    "rk_stage3": (873.3e6, _STAGE3D_SRC, "520ea50d8f39"),
 }
 
 

@@ -23,8 +23,9 @@
 //
 // Bound by instruction issue: about 75 FP32 operations and 4 reciprocals a reconstruction.
 // Against a kernel that records each face's derivatives (24 fields, 50 MB through L2 a stage on
-// 512 x 1024) and one that gathers them, the gradient of 100 steps there takes 11.45 instead of
-// 14.47 ms.  The FP64 build keeps that pair (adjoint.cuh).
+// 512 x 1024) and one that gathers them, the gradient of 100 steps there took 11.45 instead of
+// 14.47 ms; with a tile's loads sent together and the forward steps it replays made faster it
+// takes 9.2.  The FP64 build keeps that pair (adjoint.cuh).
 #pragma once
 #include "common.cuh"
 #include "weno.cuh"

@@ -19,8 +19,11 @@
 // side the face velocity comes from instead of the Lax-Friedrichs split.
 //
 // This file holds the generic one-node-per-thread form used for every lattice, precision
-// and variant; the 2D/3D FP32 production kernels live in transport_stage2d.cuh,
-// transport_sweep2d.cuh and transport_sweep3d.cuh.
+// and variant; the FP32 production kernels live in transport_tile2d.cuh (2D, lattices that
+// stay in L2), transport_stage2d_wide.cuh and transport_sweep3d_wide.cuh (larger 2D, 3D); the
+// FP64 build's 2D kernel is transport_stage2d.cuh, which LW_ONE_COLUMN (with
+// transport_sweep3d.cuh in 3D) selects in FP32, and transport_sweep2d.cuh is the
+// single-launch form.
 #pragma once
 #include "common.cuh"
 

@@ -18,9 +18,11 @@
 // instead of 12 at 133, and no priming row or half-filled wave on a small lattice; it pays with
 // halos split twice (210 instructions a node and stage instead of 186).  Bound by instruction
 // issue where the fields sit in L2 (75 % of the slots; the rest are the loads of a tile's start).
-// Whole steps, four-column kernel -> tiles: 128 x 256 15.0 -> 13.4 us, 512 x 1024 32.3 -> 24.2,
-// 1260 x 701 41.3 -> 35.8, 1024 x 2048 80.7 -> 76.3, 2048 x 2048 145.2 -> 146.4, 2048 x 4096
-// 280 -> 295.  Tiles of 64 x 16, 32 x 32 and 64 x 32 nodes were 1-5 % slower on most sizes.
+// Whole steps, four-column kernel -> tiles, the deposit folded in the same step by both:
+// 128 x 256 15.0 -> 13.4 us, 512 x 1024 32.3 -> 24.2, 1260 x 701 41.3 -> 35.8, 1024 x 2048
+// 80.7 -> 76.3, 2048 x 2048 145.2 -> 146.4, 2048 x 4096 280 -> 295 (with the fold left to the
+// next step and dependent launches 10.5, 21.5, 34.3 and 75.4 for the first four).  Tiles of
+// 64 x 16, 32 x 32 and 64 x 32 nodes were 1-5 % slower on most sizes.
 #pragma once
 #include "common.cuh"
 #include "weno.cuh"
