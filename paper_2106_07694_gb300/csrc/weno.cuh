@@ -92,9 +92,12 @@ __device__ __forceinline__ double recon_value(Recon<double> r, double c) {
   return fma(0.5, r.num * rcp_newton(r.den), c);
 }
 
-// Sum of two face values (h+ about the centre value cp, h- about cm).
+// Sum of two face values (h+ about the centre value cp, h- about cm), each rounded at its own
+// size.  Summing the two corrections first, one operation less, kept more of them than c can
+// take up a step: the drift of c against 64 bits on 128 x 256 grew by 3 % (8000 steps: 9.84e-6
+// -> 1.017e-5 relative, 9.87e-6 in this form).
 __device__ __forceinline__ float recon_sum(Recon<float> p, float cp, Recon<float> m, float cm) {
-  return fmaf(0.5f, fmaf(p.num, rcp_approx(p.den), m.num * rcp_approx(m.den)), cp + cm);
+  return fmaf(0.5f, p.num * rcp_approx(p.den), cp) + fmaf(0.5f, m.num * rcp_approx(m.den), cm);
 }
 __device__ __forceinline__ double recon_sum(Recon<double> p, double cp, Recon<double> m, double cm) {
   return fma(0.5, fma(p.num, rcp_newton(p.den), m.num * rcp_newton(m.den)), cp + cm);
