@@ -127,10 +127,10 @@ __global__ void __launch_bounds__(kAT, 4) adj_stage_kernel(Args<float> a, AdjFie
   const int nx = a.nx, ny = a.ny;
   const int x0 = blockIdx.x * kAx, y0 = blockIdx.y * kAy;
   const unsigned n = (unsigned)a.n;
-  const float* __restrict__ cs = STAGE == 3 ? a.c2 : (STAGE == 2 ? a.c1 : a.c);
-  const float* __restrict__ lsrc = STAGE == 3 ? f.mu : (STAGE == 2 ? f.lc2 : f.lc1);
-  const float* __restrict__ ux = a.u;
-  const float* __restrict__ uy = a.u + n;
+  const float* cs = STAGE == 3 ? a.c2 : (STAGE == 2 ? a.c1 : a.c);
+  const float* lsrc = STAGE == 3 ? f.mu : (STAGE == 2 ? f.lc2 : f.lc1);
+  const float* ux = a.u;
+  const float* uy = a.u + n;
   const float lscale = STAGE == 3 ? 2.f / 3.f : (STAGE == 2 ? 0.25f : 1.f);
   const float alpha = a.alpha, ia = a.inv_alpha, kappa = a.kappa, vs = a.vs;
 

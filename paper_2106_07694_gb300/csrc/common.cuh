@@ -45,10 +45,11 @@ struct Args {
 
 // Global-load policies.  LoadPlain is an ordinary load, for a kernel that may have been started
 // before the one ahead of it ended (launch_dependent): it reads what that one wrote, so the
-// read-only path is closed to it.  LoadNC reads through the non-coherent (read-only) path, for
-// data no thread writes while the kernel runs.  LoadL2 reads at L2 (ld.global.cg: no L1 line is
-// kept), for a kernel that reads what other CTAs wrote earlier in the same launch, after
-// a grid barrier.
+// read-only path is closed to it, and so is __restrict__ on its pointers, by which the compiler
+// may choose that path for an ordinary load.  LoadNC reads through the non-coherent (read-only)
+// path, for data no thread writes while the kernel runs.  LoadL2 reads at L2 (ld.global.cg: no L1
+// line is kept), for a kernel that reads what other CTAs wrote earlier in the same launch, after a
+// grid barrier.
 struct LoadNC {
   static __device__ __forceinline__ float s(const float* p) { return __ldg(p); }
   static __device__ __forceinline__ double s(const double* p) { return __ldg(p); }

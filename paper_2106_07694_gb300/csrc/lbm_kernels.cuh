@@ -203,7 +203,7 @@ __device__ __forceinline__ D2Q9Node d2q9_node(const Args<T>& a, int x, int y) {
 template <typename T, int PARITY, class LD = LoadPlain>
 __device__ __forceinline__ void d2q9_load(const Args<T>& a, const D2Q9Node& nd, T (&g)[9]) {
   const unsigned n = (unsigned)a.n;
-  const T* __restrict__ G = a.g;
+  const T* G = a.g;
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     if (PARITY == 0) {
@@ -222,7 +222,7 @@ __device__ __forceinline__ void d2q9_collide_store_c(const Args<T>& a, const D2Q
                                                      T* rho_out, const T cn) {
   const unsigned n = (unsigned)a.n;
   const unsigned node = nd.node;
-  T* __restrict__ G = a.g;
+  T* G = a.g;
   T drho = T(0), jx = T(0), jy = T(0);
 #pragma unroll
   for (int i = 0; i < 9; ++i) {

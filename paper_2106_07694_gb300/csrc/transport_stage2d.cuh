@@ -56,9 +56,9 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
   const int X = (x0 + t) % nx;
   const bool out = x0 + t < nx;
   const T inv_alpha = a.inv_alpha, vs_a = a.vs * a.inv_alpha, alpha = a.alpha, kd = a.kappa * a.inv_alpha;
-  const T* __restrict__ cin = sp.cin;
-  const T* __restrict__ ux = a.u;
-  const T* __restrict__ uy = a.u + a.n;
+  const T* cin = sp.cin;
+  const T* ux = a.u;
+  const T* uy = a.u + a.n;
 
   // staging positions of this thread in the strip + halo row (fixed for the sweep)
   const int j1 = t + kS2T;  // second position, only for the 6 halo columns

@@ -172,9 +172,9 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
   const bool out = xl < nx;
   const unsigned X = (unsigned)(xl % nx);
   const float ia = a.inv_alpha, vs_a = a.vs * a.inv_alpha, alpha = a.alpha, kd = a.kappa * a.inv_alpha;
-  const float* __restrict__ cin = sp.cin;
-  const float* __restrict__ ux = a.u;
-  const float* __restrict__ uy = a.u + a.n;
+  const float* cin = sp.cin;
+  const float* ux = a.u;
+  const float* uy = a.u + a.n;
 
   // halo quads of the staged row: thread 0 the quad left of the strip, thread 1 the one right of it
   const bool halo = t < 2;

@@ -64,9 +64,9 @@ __global__ void __launch_bounds__(kTT, 1024 / kTT) rk_tile2d_kernel(Args<float> 
   }
   const int x0 = blockIdx.x * TX, y0 = by * TY;
   const float ia = a.inv_alpha, vs_a = a.vs * a.inv_alpha, alpha = a.alpha, kd = a.kappa * a.inv_alpha;
-  const float* __restrict__ cin = sp.cin;
-  const float* __restrict__ ux = a.u;
-  const float* __restrict__ uy = a.u + a.n;
+  const float* cin = sp.cin;
+  const float* ux = a.u;
+  const float* uy = a.u + a.n;
 
   // ---- stage the tile and its halo cross
   constexpr int kQ = TX / 4 + 2, kPos = (TY + 6) * kQ;
