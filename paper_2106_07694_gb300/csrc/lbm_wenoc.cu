@@ -1,6 +1,7 @@
 // Host side of the lbm_wenoc C ABI (include/lbm_wenoc.h): parameter checks, the
 // carve-up of the caller's workspace, kernel launches, CUDA-graph replay of whole
 // steps, FP64 read-backs and per-kernel event timing.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -537,17 +538,42 @@ bool is_device_pointer(const void* p) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-// A caller's buffer that a kernel of the handle may read or write itself: ordinary device memory
-// of the handle's device, aligned to its element.  Others (host memory, another device's, a
-// managed buffer) go through a copy.
-bool kernel_can_use(const lbm_wenoc* h, const void* p) {
+// The allocation that holds p; false where the driver cannot tell.
+bool allocation_of(const void* p, uintptr_t* base, size_t* size) {
+  using Query = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const Query query = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, CUDART_VERSION, cudaEnableDefault, &found) !=
+            cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<Query>(f);
+  }();
+  CUdeviceptr b = 0;
+  if (!query || query(&b, size, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return false;
+  *base = (uintptr_t)b;
+  return true;
+}
+
+// A caller's buffer whose `bytes` a kernel of the handle may read or write itself: ordinary device
+// memory of the handle's device, aligned to its element, inside one allocation to its end and
+// outside the handle's workspace.  Others (host memory, another device's, a managed buffer, one
+// too short) go through a copy, which checks what it is given.
+bool kernel_can_use(const lbm_wenoc* h, const void* p, size_t bytes) {
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return at.type == cudaMemoryTypeDevice && at.device == h->device &&
-         reinterpret_cast<uintptr_t>(p) % (h->fp64 ? 8u : 4u) == 0;
+  const uintptr_t first = reinterpret_cast<uintptr_t>(p), ws = reinterpret_cast<uintptr_t>(h->ws);
+  if (at.type != cudaMemoryTypeDevice || at.device != h->device || first % (h->fp64 ? 8u : 4u) != 0) return false;
+  if (first < ws + h->L.total && ws < first + bytes) return false;
+  uintptr_t base = 0;
+  size_t size = 0;
+  return allocation_of(p, &base, &size) && first >= base && bytes <= size && first - base <= size - bytes;
 }
 
 // Fold the deposit of the last step where that was left to the next one.  Not only when this
@@ -715,7 +741,7 @@ int lbm_wenoc_init(lbm_wenoc* h, const void* c0, const void* u0) {
   if (cudaMemcpyAsync(h->ws + h->L.c, c0, cbytes, kc, h->stream) != cudaSuccess) return LW_ECUDA;
   const void* u0dev = nullptr;
   bool host_source = kc == cudaMemcpyHostToDevice;
-  if (u0 && kernel_can_use(h, u0)) {
+  if (u0 && kernel_can_use(h, u0, ubytes)) {
     u0dev = u0;  // read where it is
   } else if (u0) {
     cudaMemcpyKind ku = is_device_pointer(u0) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
@@ -863,8 +889,8 @@ int lbm_wenoc_fields(lbm_wenoc* h, void* rho, void* u, void* c) {
   // rho and u are computed into the caller's device buffers, or into the stage buffers (free
   // between steps) and copied out; what is not asked for is not written (except the frozen
   // velocity's rho)
-  const bool rho_direct = rho && kernel_can_use(h, rho);
-  const bool u_direct = u && !h->frozen && kernel_can_use(h, u);
+  const bool rho_direct = rho && kernel_can_use(h, rho, cbytes);
+  const bool u_direct = u && !h->frozen && kernel_can_use(h, u, cbytes * h->p.dim);
   unsigned char* rho_dev = rho_direct ? static_cast<unsigned char*>(rho) : h->ws + h->L.c2;  // free on every path
   unsigned char* u_dev = u_direct ? static_cast<unsigned char*>(u) : h->ws + h->L.u;
   if (rho || u) {
