@@ -50,7 +50,8 @@ struct AdjTileSmem {
     float y[2][kAg][8][kAx];         // ED by half, block, element (0..3 own block, 5..7 the block below), column
     float4 x[2][2][kAy][kAg];        // ED by half, own / below, row, block
   } ed;
-  float red[kAT / 32];
+  float vs_red[kAT];       // Vs terms of the threads, and of the floor nodes
+  double vs_floor[kAx];
 };
 
 // Derivatives e[0..3] of a WENO5 face value with respect to its differences d1..d4 (upwind side
@@ -110,6 +111,14 @@ __device__ __forceinline__ float column_ed(const AdjTileSmem& S, int half, int j
   float v = S.ed.y[half][b][e][col];
   if (e > 0 && b + 1 < kAg) v += S.ed.y[half][b + 1][4 + e][col];
   return v;
+}
+
+// (hi, lo) += (h, l): the rounding error of hi + h (Knuth's two-sum) is kept in lo, so a sum of
+// FP32 terms that cancel is held to about 2^-47 of their size without the narrow FP64 pipe.
+__device__ __forceinline__ void add_pair(float& hi, float& lo, float h, float l) {
+  const float s = hi + h, b = s - hi;
+  lo += l + ((hi - (s - b)) + (h - b));
+  hi = s;
 }
 
 // One stage backwards (STAGE 3, 2, 1: lambda of c', c2, c1 scaled by 2/3, 1/4, 1):
@@ -240,8 +249,8 @@ __global__ void __launch_bounds__(kAT, 4) adj_stage_kernel(Args<float> a, AdjFie
   __syncthreads();
 
   // ---- y part of the tile's nodes: four rows of one column
-  float vs_acc = 0.f;
   {
+    float vs_acc = 0.f;
     const int col = lane, r0 = 4 * warp;
     const bool own = x0 + col < nx;
     float lamF[5], edP[5], edM[5];
@@ -275,14 +284,14 @@ __global__ void __launch_bounds__(kAT, 4) adj_stage_kernel(Args<float> a, AdjFie
             vw += g;
           }
         }
-        if (own) {
-          vs_acc -= vw;
-          if (y == 0) vs_acc += c * (STAGE == 3 ? 2.f / 3.f : 1.f / 6.f) - c * S.lam[r + 4][col + 4];
-        }
+        if (own) vs_acc -= vw;
       }
       S.py[r][col] = gc;
       S.my[r][col] = gw;
     }
+    S.vs_red[tid] = vs_acc;
+    if (y0 == 0 && warp == 0)
+      S.vs_floor[col] = own ? (double)yc[0] * ((STAGE == 3 ? 2.0 / 3.0 : 1.0 / 6.0) - (double)S.lam[4][col + 4]) : 0.0;
   }
   __syncthreads();
 
@@ -382,15 +391,23 @@ __global__ void __launch_bounds__(kAT, 4) adj_stage_kernel(Args<float> a, AdjFie
     }
   }
 
-  // ---- this CTA's Vs terms
+  // ---- this CTA's Vs terms (written before the last two barriers), by one warp: the gradient of
+  // 100 steps on 512 x 1024 took 9.53 ms with the sums of a warp in plain FP32, 9.61 so, 10.03 in FP64
+  if (warp == 0) {
+    float hi = S.vs_red[lane], lo = 0.f;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) vs_acc += __shfl_down_sync(0xffffffffu, vs_acc, o);
-  if (lane == 0) S.red[warp] = vs_acc;
-  __syncthreads();
-  if (tid == 0) {
-    double s = 0.0;
-    for (int w = 0; w < kAT / 32; ++w) s += (double)S.red[w];
-    f.vs_part[blockIdx.y * gridDim.x + blockIdx.x] += s;  // own slot, fixed order over steps
+    for (int w = 1; w < kAT / 32; ++w) add_pair(hi, lo, S.vs_red[w * 32 + lane], 0.f);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      add_pair(hi, lo, __shfl_down_sync(0xffffffffu, hi, o), __shfl_down_sync(0xffffffffu, lo, o));
+    double floor_sum = 0.0;
+    if (y0 == 0) {
+      floor_sum = S.vs_floor[lane];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) floor_sum += __shfl_down_sync(0xffffffffu, floor_sum, o);
+    }
+    if (lane == 0)  // own slot, fixed order over steps
+      f.vs_part[blockIdx.y * gridDim.x + blockIdx.x] += ((double)hi + (double)lo) + floor_sum;
   }
 }
 
