@@ -22,8 +22,6 @@
 #include "common.cuh"
 #include "lattice.cuh"
 
-#include <type_traits>
-
 namespace lw {
 
 // Neighbour of (x,y,z) along direction i, sign s = +1 (x + c_i) or -1 (x - c_i).
@@ -252,28 +250,6 @@ __device__ __forceinline__ void d2q9_collide_store_c(const Args<T>& a, const D2Q
         G[i * n + (unsigned)((int)node + nd.off(i, +1))] = gs;
     }
   };
-  if constexpr (std::is_same<T, double>::value) {
-    // FP64: the step is bound by its operations, so relaxation and Guo source are taken together
-    // over the weight, in parts even and odd in c_i,
-    //   even = base + c.u (9/2 om rho c.u + 9 guo c.F),  odd = 3 om rho c.u + 3 guo c.F,
-    //   base = om (rho - 1) - 3/2 om rho u.u - 3 guo u.F:
-    // 2048 x 4096 2141 -> 1551 us.  Not in FP32, where the kernel is bound by memory (108.4 -> 105.9
-    // us) and the one rounding of base for all directions raised the error of u by a tenth.
-    const T omr = om * rho, g3 = T(3) * a.guo, g9 = T(9) * a.guo, omr3 = T(3) * omr, omr45 = T(4.5) * omr;
-    const T base = fma_t(om, drho, -fma_t(T(1.5) * omr, uu, g3 * uF));
-    store(0, fma_t(keep, g[0], T(D2Q9::w(0)) * base));
-#pragma unroll
-    for (int i = 1; i < 9; i += 2) {
-      const T wi = T(D2Q9::w(i));
-      const T cu = D2Q9::cx(i) * ux + D2Q9::cy(i) * uy;
-      const T cF = D2Q9::cx(i) * Fx + D2Q9::cy(i) * Fy;
-      const T even = wi * fma_t(cu, fma_t(omr45, cu, g9 * cF), base);
-      const T odd = fma_t(omr3, cu, g3 * cF);
-      store(i, fma_t(keep, g[i], fma_t(wi, odd, even)));
-      store(i + 1, fma_t(keep, g[i + 1], fma_t(-wi, odd, even)));
-    }
-    return;
-  }
   // rest population
   {
     const T w0 = T(D2Q9::w(0));
@@ -282,7 +258,10 @@ __device__ __forceinline__ void d2q9_collide_store_c(const Args<T>& a, const D2Q
     store(0, keep * g[0] + om * geq + src);
   }
   // opposite pairs (i, i+1) share c.u and c.F up to sign: split the equilibrium and
-  // the Guo source into parts even and odd in c_i
+  // the Guo source into parts even and odd in c_i.  Relaxation and source are rounded direction by
+  // direction: taken together over one rounded base, even = base + c.u (9/2 om rho c.u + 9 guo c.F),
+  // FP64 (bound by its operations) took 1551 instead of 2141 us on 2048 x 4096 and FP32 (bound by
+  // memory) 105.9 instead of 108.4, but u was 5 to 13 % further from the exact one in both
 #pragma unroll
   for (int i = 1; i < 9; i += 2) {
     const T wi = T(D2Q9::w(i));
