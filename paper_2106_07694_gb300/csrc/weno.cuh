@@ -29,10 +29,15 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return r;
 }
 
-// 1 / x in FP64 for positive x in the middle of the range: the hardware's approximation (a
-// relative error e0 of about 2^-20) and one third-order step of Newton's method,
-// r (1 + e + e^2) with e = 1 - x r, whose error is e0^3 < 2^-58 before rounding: four operations
-// with the product, where an IEEE division takes about ten of the narrow FP64 pipe.
+// 1 / x in FP64 for the weights' denominators, positive and from 10 (3/4 1e-6)^4 = 3e-24 up: the
+// hardware's approximation, of relative error e0, and one step r (1 + e + e^2) with e = 1 - x r,
+// the third-order hyperpower iteration for an inverse (Altman 1960).  x r (1 + e + e^2) =
+// (1 - e)(1 + e + e^2) = 1 - e^3, so e0^3 is left beside the last rounding: with e0 of 2^-20 under
+// 0.51 units in the last place (tested: within one unit of IEEE division from 3e-24 to 1e60, the
+// quotient within two).  Four operations with the product, where an IEEE division takes about ten
+// of the narrow FP64 pipe: a step on 128 x 256 takes 68.6 us, 74.9 with divisions.  c and u are no
+// further from a long-double run with it (300 x 133 after 1500 steps: c 3.98e-14 both, 128 x 256
+// after 8000: 2.76e-14 both; with division and the 12/13 form of the indicators 3.98e-14, 2.79e-14).
 __device__ __forceinline__ double rcp_newton(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -99,6 +104,9 @@ __device__ __forceinline__ double recon_value(Recon<double> r, double c) {
 __device__ __forceinline__ float recon_sum(Recon<float> p, float cp, Recon<float> m, float cm) {
   return fmaf(0.5f, p.num * rcp_approx(p.den), cp) + fmaf(0.5f, m.num * rcp_approx(m.den), cm);
 }
+// In FP64, where the pipe is narrow, the corrections are summed first: a face is then 6e-18 from the
+// exact one (rms on a noisy front) against 2.7e-17, and over 8000 steps c drifts no more than with
+// the values rounded one by one (2.758e-14 against 2.761e-14).
 __device__ __forceinline__ double recon_sum(Recon<double> p, double cp, Recon<double> m, double cm) {
   return fma(0.5, fma(p.num, rcp_newton(p.den), m.num * rcp_newton(m.den)), cp + cm);
 }
