@@ -180,11 +180,11 @@ int lbm_wenoc_profile_read(lbm_wenoc* h, lbm_wenoc_kernel_stat* out, int max, in
 /* Number of kernel launches this handle has issued since create. */
 int64_t lbm_wenoc_launch_count(const lbm_wenoc* h);
 
-/* Tuning of the FP32 transport sweeps: rows per CTA segment of the 2D stage kernels (or
- * of the fused 2D kernel), or z levels per CTA segment of the 3D stage kernels (0 = default).  Results do not
- * depend on it (bitwise).  No effect on 3D FP64 or periodic-vertical handles, nor on the 2D FP32
- * lattices small enough to run on tiles (3.5 M nodes).  Drops
- * captured graphs; call between steps. */
+/* Tuning of the transport sweeps: rows per CTA segment of the 2D stage kernels (or of the
+ * fused 2D kernel), or z levels per CTA segment of the 3D stage kernels (0 = default).  A
+ * positive height also takes a 2D FP32 lattice small enough to run on tiles (3.5 M nodes) to
+ * the row sweep, 0 takes it back.  Results do not depend on it (bitwise).  No effect on 3D
+ * FP64 or periodic-vertical handles.  Drops captured graphs; call between steps. */
 int lbm_wenoc_set_segment_rows(lbm_wenoc* h, int32_t rows);
 
 /* ---- Batched simulations (the paper's parameter sweep, Sec. 2.2 Table 1, as one job) ----

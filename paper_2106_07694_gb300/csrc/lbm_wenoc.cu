@@ -145,8 +145,9 @@ struct lbm_wenoc {
   bool stage2d = false;  // 2D FP32 with walls: three row-sweep stage kernels
   int stage2d_rows = 0;
   bool wide = false;     // ... with four columns per thread (FP32, without LW_ONE_COLUMN)
-  bool tile = false;     // ... on tiles (four-column handles whose lattice stays in L2)
-  int late_count = 0;    // partials of the deposit folded late (0: the last stage folds them)
+  bool tiles_fit = false;  // four-column handles whose lattice stays in L2
+  bool tile = false;     // ... run on tiles: tiles_fit, and no segment height was asked for
+  int late_slots = 0;    // partials of the deposit that a step on tiles leaves to the next (0: it folds them)
   bool late_pending = false;  // a step of this handle since the last fold
   int wide_per_sm = 1;   // CTAs of the four-column stage kernel one SM holds at once
   bool initialised = false;
@@ -208,7 +209,7 @@ Args<T> make_args(const lbm_wenoc* h) {
   a.inv_alpha = T(1.0 / h->alpha);
   a.u_cap = T(p.u_cap);
   a.scheme = scheme_bits(p);
-  a.late_count = h->late_count;
+  a.late_count = h->tile ? h->late_slots : 0;
   if (h->sugar) {
     a.S = reinterpret_cast<T*>(b + (h->cur ? h->L.sb : h->L.sa));
     a.S2 = reinterpret_cast<T*>(b + (h->cur ? h->L.sa : h->L.sb));
@@ -580,9 +581,10 @@ bool kernel_can_use(const lbm_wenoc* h, const void* p, size_t bytes) {
 // handle knows of a step since the last fold: steps that a caller captured into a graph of its own
 // are replayed without it.  With nothing left the partials are zero.
 int fold_late(lbm_wenoc* h) {
-  if (h->late_count == 0) return LW_OK;
+  if (h->late_slots == 0) return LW_OK;
   h->late_pending = false;
-  const Args<float> a = make_args<float>(h);  // FP32 handles only
+  Args<float> a = make_args<float>(h);  // FP32 handles only
+  a.late_count = h->late_slots;
   lw::late_deposit_kernel<float><<<1, 32, 0, h->stream>>>(a);
   return cudaGetLastError() == cudaSuccess ? LW_OK : LW_ECUDA;
 }
@@ -671,7 +673,7 @@ int lbm_wenoc_create(const lbm_wenoc_params* p, void* dev_workspace, size_t byte
   // (FP64 too: the validation build runs the one-column form)
   h->stage2d = h->p.dim == 2 && h->walls && !h->sweep && (p->nx + lw::kS2T - 1) / lw::kS2T <= lw::kMaxReduceBlocks;
   h->wide = h->stage2d && !h->fp64 && !(p->flags & LW_ONE_COLUMN);
-  h->tile = h->wide && lw::tile2d_use(p->nx, p->ny);
+  h->tile = h->tiles_fit = h->wide && lw::tile2d_use(p->nx, p->ny);
   if (h->stage2d) {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess || sms <= 0) sms = 148;
@@ -721,7 +723,7 @@ int lbm_wenoc_create(const lbm_wenoc_params* p, void* dev_workspace, size_t byte
   // on tiles the deposit of a step is folded by the next step (one class: the classes share the
   // partials, one after the other)
   if (h->tile && h->ncls == 1 && (p->nx + lw::kTX - 1) / lw::kTX <= lw::kLateMax)
-    h->late_count = (p->nx + lw::kTX - 1) / lw::kTX;
+    h->late_slots = (p->nx + lw::kTX - 1) / lw::kTX;
   h->kind_names.assign(kKindNames, kKindNames + K_COUNT);
   h->kind_launches.assign(K_COUNT, 0);
   h->kind_ms.assign(K_COUNT, 0.0);
@@ -785,7 +787,7 @@ int lbm_wenoc_step(lbm_wenoc* h, int64_t nsteps) {
   if (!h || nsteps < 0) return LW_EINVAL;
   if (!h->initialised) return LW_ESTATE;
   int64_t left = nsteps;
-  if (nsteps > 0) h->late_pending = h->late_count > 0;
+  if (nsteps > 0 && h->tile) h->late_pending = h->late_slots > 0;
   if (h->use_graphs && !h->profiling) {
     while (left > 0) {
       const int par = h->frozen ? 0 : h->parity;
@@ -1149,6 +1151,11 @@ int lbm_wenoc_set_segment_rows(lbm_wenoc* h, int32_t rows) {
     if (h->stage2d)
       h->stage2d_rows = h->wide ? lw::stage2d_wide_rows(h->p.nx, h->p.ny, sms, h->wide_per_sm, rows)
                                 : lw::stage2d_rows(h->p.nx, h->p.ny, sms, rows);
+    if (h->tiles_fit) {  // tiles have no segments: a height selects the row sweep, which leaves no partials
+      if (h->initialised)
+        if (int rc = fold_late(h)) return rc;
+      h->tile = rows == 0;
+    }
     return LW_OK;
   }
   if (!h->sweep) return LW_OK;
@@ -1699,7 +1706,7 @@ int record_step(lbm_wenoc* h, const StepRecord<T>& R, bool first, T* next) {
   a.c1 = R.c1;
   a.c2 = R.c2;
   a.u = R.u;
-  h->late_pending = h->late_count > 0;
+  if (h->tile) h->late_pending = h->late_slots > 0;
   const dim3 blk(kLbmThreads), grd((a.nx + kLbmThreads - 1) / kLbmThreads, a.ny, 1);
   launch(h, K_LBM, [&] {
     if (h->parity == 0)
