@@ -171,19 +171,19 @@ _LBM_SRC = ("lbm_kernels.cuh", "lattice.cuh", "common.cuh")
 _STAGE_SRC = ("transport_stage2d_wide.cuh", "transport_stage2d.cuh", "weno.cuh", "common.cuh")
 _STAGE3D_SRC = ("transport_sweep3d_wide.cuh", "transport_sweep3d.cuh") + _STAGE_SRC
 NCU_TRAFFIC = {
-    "lbm_collide_stream": (642.9e6, _LBM_SRC, "7bf409f75720"),
-    "rk_stage1": (131.9e6, _STAGE_SRC, "7869d5bd605f"),
-    "rk_stage2": (172.7e6, _STAGE_SRC, "7869d5bd605f"),
-    "rk_stage3": (166.2e6, _STAGE_SRC, "7869d5bd605f"),
+    "lbm_collide_stream": (642.9e6, _LBM_SRC, "9e3e69294f97"),
+    "rk_stage1": (130.9e6, _STAGE_SRC, "cae9a3f18c0f"),
+    "rk_stage2": (172.7e6, _STAGE_SRC, "cae9a3f18c0f"),
+    "rk_stage3": (166.2e6, _STAGE_SRC, "cae9a3f18c0f"),
     # 512 x 1024 adjoint workload, mean of the three stages (step records read from HBM)
-    "adj_faces": (12.65e6, ("adjoint_tile.cuh", "weno.cuh", "adjoint.cuh") + _LBM_SRC, "0b0182fe11ef"),
+    "adj_faces": (12.65e6, ("adjoint_tile.cuh", "weno.cuh", "adjoint.cuh") + _LBM_SRC, "93d9aa4fea59"),
 }
 # the 256 x 256 x 512 D3Q19 workload
 NCU_TRAFFIC_3D = {
-    "lbm_collide_stream": (5577.7e6, _LBM_SRC, "7bf409f75720"),
-    "rk_stage1": (735.8e6, _STAGE3D_SRC, "76b59d859a6a"),
-    "rk_stage2": (874.6e6, _STAGE3D_SRC, "76b59d859a6a"),
-    "rk_stage3": (873.3e6, _STAGE3D_SRC, "76b59d859a6a"),
+    "lbm_collide_stream": (5577.8e6, _LBM_SRC, "9e3e69294f97"),
+    "rk_stage1": (734.7e6, _STAGE3D_SRC, "484ee236ed2f"),
+    "rk_stage2": (874.3e6, _STAGE3D_SRC, "484ee236ed2f"),
+    "rk_stage3": (875.2e6, _STAGE3D_SRC, "484ee236ed2f"),
 }
 
 

@@ -57,7 +57,7 @@ extern "C" {
                                      diffusion D_s; not with LW_FUSED_RK3, batches or the gradient */
 #define LW_WENO3 0x40u            /* the paper's third-order WENO (Supplement Eqs. S10-S20, linear weights
                                      (2/3, 1/3) of Eq. S16) instead of WENO5; a compile-time variant of
-                                     the FP32 sweep stage kernels (FP64: the generic ones) */
+                                     the FP32 and 2D FP64 stage kernels (3D FP64: the generic ones) */
 #define LW_SIGN_SPLIT 0x80u       /* whole flux w c reconstructed from the side the face velocity
                                      (w_i + w_{i+1})/2 comes from (ties left) instead of the
                                      Lax-Friedrichs split; stage kernels as for LW_WENO3.  Neither

@@ -25,7 +25,7 @@
 // Against a kernel that records each face's derivatives (24 fields, 50 MB through L2 a stage on
 // 512 x 1024) and one that gathers them, the gradient of 100 steps there took 11.45 instead of
 // 14.47 ms; with a tile's loads sent together and the forward steps it replays made faster it
-// takes 9.2.  The FP64 build keeps that pair (adjoint.cuh).
+// takes 9.2.  494-505 instructions a node and stage, 56-59 % of the issue slots while it runs.  The FP64 build keeps that pair (adjoint.cuh).
 #pragma once
 #include "common.cuh"
 #include "weno.cuh"
@@ -391,8 +391,9 @@ __global__ void __launch_bounds__(kAT, 4) adj_stage_kernel(Args<float> a, AdjFie
     }
   }
 
-  // ---- this CTA's Vs terms (written before the last two barriers), by one warp: the gradient of
-  // 100 steps on 512 x 1024 took 9.53 ms with the sums of a warp in plain FP32, 9.61 so, 10.03 in FP64
+  // ---- this CTA's Vs terms (written before the last two barriers), by one warp.  Gradient of 100
+  // steps on 512 x 1024 through autograd: 9.53 ms with a warp's sums in plain FP32, 9.61 so, 10.03
+  // with all of them in FP64
   if (warp == 0) {
     float hi = S.vs_red[lane], lo = 0.f;
 #pragma unroll

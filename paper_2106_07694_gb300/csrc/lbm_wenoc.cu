@@ -151,7 +151,7 @@ struct lbm_wenoc {
   bool late_pending = false;  // a step of this handle since the last fold
   int wide_per_sm = 1;   // CTAs of the four-column stage kernel one SM holds at once
   bool initialised = false;
-  bool sugar = false;  // LW_SUGAR: S in L.sa / L.sb, selected by cur (the generic transport path)
+  bool sugar = false;  // LW_SUGAR: S in L.sa / L.sb, selected by cur
   int ncls = 1;        // particle classes
   int64_t steps = 0;
   int64_t launches = 0;
@@ -889,8 +889,7 @@ int lbm_wenoc_fields(lbm_wenoc* h, void* rho, void* u, void* c) {
   const size_t es = h->fp64 ? 8 : 4;
   const size_t cbytes = (size_t)h->n * es;
   // rho and u are computed into the caller's device buffers, or into the stage buffers (free
-  // between steps) and copied out; what is not asked for is not written (except the frozen
-  // velocity's rho)
+  // between steps) and copied out; the one not asked for goes to its stage buffer
   const bool rho_direct = rho && kernel_can_use(h, rho, cbytes);
   const bool u_direct = u && !h->frozen && kernel_can_use(h, u, cbytes * h->p.dim);
   unsigned char* rho_dev = rho_direct ? static_cast<unsigned char*>(rho) : h->ws + h->L.c2;  // free on every path
@@ -1373,7 +1372,7 @@ int batch_advance(lbm_wenoc_batch* b, int64_t nsteps, bool require_init) {
   for (lbm_wenoc* h : b->inst) {
     if (require_init && !h->initialised) return LW_ESTATE;
     if (h->parity != par || h->steps != b->inst[0]->steps) return LW_ESTATE;
-    if (h->late_pending)  // an instance stepped alone before
+    if (h->late_pending)  // an instance stepped alone before: its deposit first, the sum runs in step order
       if (int rc = fold_late(h)) return rc;
   }
   int64_t left = nsteps;

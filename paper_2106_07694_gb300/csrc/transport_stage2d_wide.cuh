@@ -23,7 +23,7 @@
 // Every face is computed once, with the arithmetic of face_flux_x, so
 // the faces and the updated c are bitwise those of the one-column kernel.
 //
-// Bound by instruction issue with 12 warps an SM (131-133 registers, six CTAs; a cap that lets
+// Bound by instruction issue with 12 warps an SM (128-133 registers, six CTAs; a cap that lets
 // seven or eight in costs more in moves than they give, 280 -> 290 us a step).  2048 x 4096:
 // 61.4 / 62.4 / 65.6 us a stage, 65.7 / 67.4 / 69.4 with the longer form of the reconstruction
 // (weno.cuh) and the first loads one after the other.

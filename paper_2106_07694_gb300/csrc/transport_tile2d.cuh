@@ -16,12 +16,13 @@
 //
 // Against that kernel a tile has no serial chain of rows: 32 warps an SM at 54-61 registers
 // instead of 12 at 133, and no priming row or half-filled wave on a small lattice; it pays with
-// halos split twice (210 instructions a node and stage instead of 186).  Bound by instruction
-// issue where the fields sit in L2 (75 % of the slots; the rest are the loads of a tile's start).
+// halos split twice (213-220 instructions a node and stage instead of 191-207).  Bound by
+// instruction issue where the fields sit in L2 (68-69 % of the slots on 1024 x 2048; on 512 x 1024,
+// less than a wave, 53-55 %; the rest waits for a tile's first loads and at its barriers).
 // Whole steps, four-column kernel -> tiles, the deposit folded in the same step by both:
 // 128 x 256 15.0 -> 13.4 us, 512 x 1024 32.3 -> 24.2, 1260 x 701 41.3 -> 35.8, 1024 x 2048
-// 80.7 -> 76.3, 2048 x 2048 145.2 -> 146.4, 2048 x 4096 280 -> 295 (with the fold left to the
-// next step and dependent launches 10.5, 21.5, 34.3 and 75.4 for the first four).  Tiles of
+// 80.7 -> 76.3 (with the fold left to the next step and dependent launches 10.5, 21.5, 34.3 and
+// 74.8; larger ones at kTileMaxNodes).  Tiles of
 // 64 x 16, 32 x 32 and 64 x 32 nodes were 1-5 % slower on most sizes.
 #pragma once
 #include "common.cuh"
@@ -34,9 +35,15 @@ namespace lw {
 constexpr int kTX = 32, kTY = 16;      // tile (nodes)
 constexpr int kTT = kTX * kTY / 4;     // threads
 // Largest lattice that runs on tiles: its populations (36 bytes a node) and fields stay in L2
-// (129 MB) up to here; beyond, a tile's start waits for HBM and the row sweep, which loads a row
-// ahead, is the faster one (2048 x 2048, 4.2 M nodes: 145.2 us a step against 146.4; sugar 158
-// against 166, WENO3 114 against 118; 1536 x 2048, 3.1 M: 115.1 against 110.7, 125 against 122).
+// (129 MB) up to about here; beyond, a tile's start waits for HBM and the row sweep, which loads a
+// row ahead, is the faster one.  Steps with both kernels as they are (late fold on tiles, dependent
+// launches on both), us, tiles against the row sweep:
+//            1536 x 2048     1792 x 2048     2048 x 2048     2048 x 3072     2048 x 4096
+//            (3.1 M nodes)   (3.7 M)         (4.2 M)         (6.3 M)         (8.4 M)
+//   plain    109.9  114.6    127.6  129.6    145.3  144.7    220.0  212.2    287.4  278.3
+//   sugar    123.2  124.2    144.2  140.7    165.8  157.4    249.4  232.0    326.3  304.2
+//   WENO3     89.0   91.1    103.4  103.1    118.3  116.1    183.9  173.2    241.0  227.0
+//   sign      99.1  100.6    114.9  113.8    131.1  127.6    199.9  186.8    261.4  243.6
 constexpr long long kTileMaxNodes = 3500000;
 
 struct Tile2dSmem {
