@@ -24,6 +24,8 @@
 // binary search in the prefix table of block counts and runs the single-instance body.
 // All forms run the same per-node arithmetic as the single-instance kernels.
 #pragma once
+#include <cmath>
+
 #include "common.cuh"
 #include "lbm_kernels.cuh"
 #include "transport_stage2d_wide.cuh"
@@ -287,6 +289,40 @@ __global__ void __launch_bounds__(kWT, kPersistMinB) batch_persistent_kernel(Bat
     batch_stage_phase<3>(t, t.queue + 3 * k + 2, S, sa, s_inst, s_meta);
     if (k + 1 < nsteps && !batch_grid_sync(t, nb, wait_limit, s_ok)) return;
   }
+}
+
+// Rows per segment of a batch's stage items, one height for all of them, over `grid` CTAs that take
+// items as they come; an item of H rows costs about H + 2 (ring fill, priming row).
+// With many items the last ones end H + 2 rows apart, half of that on average: N / (256 grid)
+// (1 + 2/H) + (H + 2)/2 rows for N nodes, least at H = 2 sqrt(N / (256 grid)).  64 instances, 56 M
+// nodes: 27; a step takes 2.52 ms with each instance's own height for a run alone (2 to 20 rows,
+// sized to fill the chip by itself), 2.23 ms at 32 rows, 2.25 at 48, 2.29 at 64.
+// With few the last wave's emptiness counts, so they take the height of the least waves x (H + 2).
+// Grouped launch, us a step, rule for many -> waves: one 1024 x 2048 107 -> 94, one 2048 x 4096
+// 343 -> 315, five of 256..1024 x 512..2048 206 -> 176, 16 of them 771 -> 741 (4.1 waves), 32 the same;
+// persistent 122 -> 118, 360 -> 344, 211 -> 197, 774 -> 765.
+constexpr int kBatchFewWaves = 5;
+inline int batch_rows(const int* nx, const int* ny, int count, long long grid) {
+  double nodes = 0.0;
+  for (int i = 0; i < count; ++i) nodes += (double)nx[i] * ny[i];
+  auto items = [&](int H) {
+    long long n = 0;
+    for (int i = 0; i < count; ++i) n += (long long)((nx[i] + kWW - 1) / kWW) * ((ny[i] + H - 1) / H);
+    return n;
+  };
+  const int root = (int)(2.0 * std::sqrt(nodes / ((double)kWW * (double)grid)) + 0.5);
+  const int many = root < 2 ? 2 : root > kWmaxH ? kWmaxH : root;
+  if (items(many) > kBatchFewWaves * grid) return many;
+  int best = 2;
+  long long best_cost = -1;
+  for (int H = 2; H <= kWmaxH; ++H) {
+    const long long cost = (items(H) + grid - 1) / grid * (H + 2);
+    if (best_cost < 0 || cost < best_cost) {
+      best_cost = cost;
+      best = H;
+    }
+  }
+  return best;
 }
 
 }  // namespace lw

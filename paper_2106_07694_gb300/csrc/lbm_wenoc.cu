@@ -1227,18 +1227,14 @@ void batch_destroy_graphs(lbm_wenoc_batch* b) {
   }
 }
 
-// Rows per segment of the stage items unless the autotuner chose others, one height for the
-// whole batch.  With N nodes over `grid` CTAs that take items as they come, an item of H rows
-// costs about H + 2 (ring fill, priming row) and the last ones end H + 2 rows apart, half of
-// that on average: N / (256 grid) (1 + 2/H) + (H + 2)/2 rows, least at H = 2 sqrt(N / (256 grid)).
-// 64 instances, 56 M nodes: 27; a step takes 2.52 ms with each instance's own height for a run
-// alone (2 to 20 rows, sized to fill the chip by itself), 2.23 ms at 32 rows, 2.25 at 48, 2.29
-// at 64.
+// Rows per segment of the stage items unless the autotuner chose others.
 int batch_default_rows(const lbm_wenoc_batch* b) {
-  double nodes = 0.0;
-  for (const lbm_wenoc* h : b->inst) nodes += (double)h->n;
-  const double per = nodes / ((double)lw::kWW * std::max(1, b->grid));
-  return std::max(2, std::min(lw::kWmaxH, (int)std::lround(2.0 * std::sqrt(per))));
+  std::vector<int> nx, ny;
+  for (const lbm_wenoc* h : b->inst) {
+    nx.push_back(h->p.nx);
+    ny.push_back(h->p.ny);
+  }
+  return lw::batch_rows(nx.data(), ny.data(), (int)b->inst.size(), std::max(1, b->grid));
 }
 
 // Fill the device tables from the instances' current argument blocks and geometries.
