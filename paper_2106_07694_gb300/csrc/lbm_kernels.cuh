@@ -452,6 +452,8 @@ __global__ void __launch_bounds__(128) init_kernel(Args<T> a, const T* u0) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y;
   const int z = blockIdx.z;
+  if (x < a.late_count && y == 0 && z == 0)  // no deposit left to fold: at most a partial per 32 columns
+    a.partials[kLateOffset + x] = 0.0;
   if (x >= a.nx) return;
   const long long n = a.n;
   const long long node = ((long long)z * a.ny + y) * a.nx + x;

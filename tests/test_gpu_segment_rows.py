@@ -133,3 +133,17 @@ def test_replayed_tile_steps_count_after_a_switch():
     with torch.cuda.stream(ref.stream):
         ref.step(2)
     assert s.deposit == ref.deposit > 0
+
+
+@pytest.mark.parametrize("shape,rows", [((4, 8), 0), ((260, 40), 0), ((260, 40), 6), ((2308, 16), 0)])
+def test_a_fresh_state_drops_what_a_step_left(shape, rows):
+    s, ref = (lw.Simulation(shape, **KW) for _ in range(2))
+    _init(s, shape, {})
+    s.step(5)
+    lw.lbm_wenoc_set_segment_rows(s.handle, rows)
+    for k in (s, ref):
+        _init(k, shape, {})
+    assert s.deposit == 0.0
+    for k in (s, ref):
+        k.step(3)
+    assert s.deposit == ref.deposit > 0
