@@ -202,9 +202,9 @@ __device__ __forceinline__ void stage2d_body(const Args<T>& a, const Stage2dPara
     if (!prime) {
       const T vs_floor = SUGAR && k == 0 ? a.vs * fma_t(-a.ks, LoadPlain::s(a.S + X), T(1)) : a.vs;
       const T Lk = S.fx[t] - S.fx[t == kS2T - 1 && !edge ? 0 : t + 1] + (carry - fup);  // carry is 0 below the floor row
-      const T cb = k == 0 ? fma_t(-vs_floor, chere, chere) : chere;  // less the floor outflow
       if (out) {
-        const T v = rk_combine<STAGE>(cb, Lk, alpha, cn_here);
+        const T v = k == 0 ? rk_combine_floor<STAGE>(chere, Lk, alpha, cn_here, vs_floor)
+                           : rk_combine<STAGE>(chere, Lk, alpha, cn_here);
         sp.cout[(unsigned)k * (unsigned)nx + X] = v;
         if (STAGE == 3) {
           report_status(a.status, !isfinite(v));

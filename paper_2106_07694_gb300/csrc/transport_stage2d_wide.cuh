@@ -350,7 +350,9 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
       const float ch[4] = {cq.x, cq.y, cq.z, cq.w};
       const float cnv[4] = {cn.x, cn.y, cn.z, cn.w};
       const float cy[4] = {carry.x, carry.y, carry.z, carry.w};
-      float v[4], cb[4] = {ch[0], ch[1], ch[2], ch[3]};
+      float v[4], Lk[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) Lk[j] = fxq[j] - fr[j] + (cy[j] - fup[j]);
       float vsf[4] = {a.vs, a.vs, a.vs, a.vs};
       if (k == 0) {  // the floor row's settling outflow (its lower face, carry, is 0)
         if (SUGAR) {
@@ -361,10 +363,12 @@ __device__ __forceinline__ void stage2d_wide_body(StageWideSmem& S, const Args<f
           vsf[3] *= fmaf(-a.ks, s0.w, 1.f);
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) cb[j] = fmaf(-vsf[j], ch[j], ch[j]);
-      }
+        for (int j = 0; j < 4; ++j)
+          v[j] = rk_combine_floor<STAGE>(ch[j], Lk[j], alpha, cnv[j], vsf[j]);
+      } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = rk_combine<STAGE>(cb[j], fxq[j] - fr[j] + (cy[j] - fup[j]), alpha, cnv[j]);
+        for (int j = 0; j < 4; ++j) v[j] = rk_combine<STAGE>(ch[j], Lk[j], alpha, cnv[j]);
+      }
       if (out) {
         *reinterpret_cast<float4*>(sp.cout + (unsigned)k * (unsigned)nx + X) = make_float4(v[0], v[1], v[2], v[3]);
         if (STAGE == 3) {

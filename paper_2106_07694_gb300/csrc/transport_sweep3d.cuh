@@ -236,10 +236,10 @@ __device__ __forceinline__ void rk_sweep3d_body(const Args<float>& a, const Swee
     if (!prime) {
       const float vs_floor = SUGAR && k == 0 ? a.vs * fmaf(-a.ks, __ldg(a.S + col), 1.f) : a.vs;
       const float Lk = S.fx[ty][tx] - S.fx[ty][tx + 1] + S.fy[ty][tx] - S.fy[ty + 1][tx] + carry - fup;
-      const float cb = k == 0 ? fmaf(-vs_floor, chere, chere) : chere;  // less the floor outflow (carry is 0 there)
       if (out) {
         const unsigned node = lv + col;
-        const float v = rk_combine<STAGE>(cb, Lk, alpha, cn_here);
+        const float v = k == 0 ? rk_combine_floor<STAGE>(chere, Lk, alpha, cn_here, vs_floor)  // carry is 0 there
+                               : rk_combine<STAGE>(chere, Lk, alpha, cn_here);
         sp.cout[node] = v;
         if (STAGE == 3) report_status(a.status, !isfinite(v));
       }

@@ -298,7 +298,9 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
       const float ch[4] = {cq.x, cq.y, cq.z, cq.w};
       const float cnv[4] = {cn.x, cn.y, cn.z, cn.w};
       const float cy[4] = {carry.x, carry.y, carry.z, carry.w};
-      float v[4], cb[4] = {ch[0], ch[1], ch[2], ch[3]};
+      float v[4], Lk[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) Lk[j] = fxq[j] - fr[j] + fyl4[j] - fyu4[j] + cy[j] - fup[j];
       if (k == 0) {  // the floor level's settling outflow (its lower face, carry, is 0)
         float vsf[4] = {a.vs, a.vs, a.vs, a.vs};
         if (SUGAR) {
@@ -309,11 +311,11 @@ __device__ __forceinline__ void sweep3d_wide_body(Sweep3dWideSmem& S, const Args
           vsf[3] *= fmaf(-a.ks, s0.w, 1.f);
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) cb[j] = fmaf(-vsf[j], ch[j], ch[j]);
-      }
+        for (int j = 0; j < 4; ++j) v[j] = rk_combine_floor<STAGE>(ch[j], Lk[j], alpha, cnv[j], vsf[j]);
+      } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        v[j] = rk_combine<STAGE>(cb[j], fxq[j] - fr[j] + fyl4[j] - fyu4[j] + cy[j] - fup[j], alpha, cnv[j]);
+        for (int j = 0; j < 4; ++j) v[j] = rk_combine<STAGE>(ch[j], Lk[j], alpha, cnv[j]);
+      }
       if (out) {
         *reinterpret_cast<float4*>(sp.cout + (unsigned)k * plane + col) = make_float4(v[0], v[1], v[2], v[3]);
         if (STAGE == 3)

@@ -196,7 +196,9 @@ __global__ void __launch_bounds__(kTT, 1024 / kTT) rk_tile2d_kernel(Args<float> 
     const float4 dy = *reinterpret_cast<const float4*>(&S.py[row][4 * q]);
     const float frq[4] = {fxq[1], fxq[2], fxq[3], fr};
     const float ch[4] = {cq.x, cq.y, cq.z, cq.w}, cnv[4] = {cn.x, cn.y, cn.z, cn.w}, dyv[4] = {dy.x, dy.y, dy.z, dy.w};
-    float v[4], cb[4] = {ch[0], ch[1], ch[2], ch[3]};
+    float v[4], Lk[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) Lk[j] = fxq[j] - frq[j] + dyv[j];
     float vsf[4] = {a.vs, a.vs, a.vs, a.vs};
     if (y == 0) {  // the floor row's settling outflow
       if (SUGAR) {
@@ -207,10 +209,12 @@ __global__ void __launch_bounds__(kTT, 1024 / kTT) rk_tile2d_kernel(Args<float> 
         vsf[3] *= fmaf(-a.ks, s0.w, 1.f);
       }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) cb[j] = fmaf(-vsf[j], ch[j], ch[j]);
-    }
+      for (int j = 0; j < 4; ++j)
+        v[j] = rk_combine_floor<STAGE>(ch[j], Lk[j], alpha, cnv[j], vsf[j]);
+    } else {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = rk_combine<STAGE>(cb[j], fxq[j] - frq[j] + dyv[j], alpha, cnv[j]);
+      for (int j = 0; j < 4; ++j) v[j] = rk_combine<STAGE>(ch[j], Lk[j], alpha, cnv[j]);
+    }
     *reinterpret_cast<float4*>(sp.cout + node) = make_float4(v[0], v[1], v[2], v[3]);
     if (STAGE == 3) {
       report_status(a.status, !(isfinite(v[0]) && isfinite(v[1]) && isfinite(v[2]) && isfinite(v[3])));

