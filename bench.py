@@ -171,19 +171,19 @@ _LBM_SRC = ("lbm_kernels.cuh", "lattice.cuh", "common.cuh")
 _STAGE_SRC = ("transport_stage2d_wide.cuh", "transport_stage2d.cuh", "weno.cuh", "common.cuh")
 _STAGE3D_SRC = ("transport_sweep3d_wide.cuh", "transport_sweep3d.cuh") + _STAGE_SRC
 NCU_TRAFFIC = {
-    "lbm_collide_stream": (642.9e6, _LBM_SRC, "dcbefe5df18d"),
-    "rk_stage1": (130.9e6, _STAGE_SRC, "cae9a3f18c0f"),
-    "rk_stage2": (172.7e6, _STAGE_SRC, "cae9a3f18c0f"),
-    "rk_stage3": (166.2e6, _STAGE_SRC, "cae9a3f18c0f"),
+    "lbm_collide_stream": (643.0e6, _LBM_SRC, "dcbefe5df18d"),
+    "rk_stage1": (131.6e6, _STAGE_SRC, "df81c1304f23"),
+    "rk_stage2": (172.9e6, _STAGE_SRC, "df81c1304f23"),
+    "rk_stage3": (166.3e6, _STAGE_SRC, "df81c1304f23"),
     # 512 x 1024 adjoint workload, mean of the three stages (step records read from HBM)
-    "adj_faces": (12.65e6, ("adjoint_tile.cuh", "weno.cuh", "adjoint.cuh") + _LBM_SRC, "9d77c269412a"),
+    "adj_faces": (12.65e6, ("adjoint_tile.cuh", "weno.cuh", "adjoint.cuh") + _LBM_SRC, "c9d11db0bd52"),
 }
 # the 256 x 256 x 512 D3Q19 workload
 NCU_TRAFFIC_3D = {
-    "lbm_collide_stream": (5577.8e6, _LBM_SRC, "dcbefe5df18d"),
-    "rk_stage1": (734.7e6, _STAGE3D_SRC, "484ee236ed2f"),
-    "rk_stage2": (874.3e6, _STAGE3D_SRC, "484ee236ed2f"),
-    "rk_stage3": (875.2e6, _STAGE3D_SRC, "484ee236ed2f"),
+    "lbm_collide_stream": (5577.9e6, _LBM_SRC, "dcbefe5df18d"),
+    "rk_stage1": (736.0e6, _STAGE3D_SRC, "3d112c409c5c"),
+    "rk_stage2": (874.2e6, _STAGE3D_SRC, "3d112c409c5c"),
+    "rk_stage3": (875.2e6, _STAGE3D_SRC, "3d112c409c5c"),
 }
 
 

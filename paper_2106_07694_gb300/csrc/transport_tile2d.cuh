@@ -18,7 +18,7 @@
 // instead of 12 at 133, and no priming row or half-filled wave on a small lattice; it pays with
 // halos split twice (213-220 instructions a node and stage instead of 191-207).  Bound by
 // instruction issue where the fields sit in L2 (68-69 % of the slots on 1024 x 2048; on 512 x 1024,
-// less than a wave, 53-55 %; the rest waits for a tile's first loads and at its barriers).
+// less than a wave, 52 %; the rest waits for a tile's first loads and at its barriers).
 // Whole steps, four-column kernel -> tiles, the deposit folded in the same step by both:
 // 128 x 256 15.0 -> 13.4 us, 512 x 1024 32.3 -> 24.2, 1260 x 701 41.3 -> 35.8, 1024 x 2048
 // 80.7 -> 76.3 (with the fold left to the next step and dependent launches 10.5, 21.5, 34.3 and
@@ -40,10 +40,10 @@ constexpr int kTT = kTX * kTY / 4;     // threads
 // launches on both), us, tiles against the row sweep:
 //            1536 x 2048     1792 x 2048     2048 x 2048     2048 x 3072     2048 x 4096
 //            (3.1 M nodes)   (3.7 M)         (4.2 M)         (6.3 M)         (8.4 M)
-//   plain    109.9  114.6    127.6  129.6    145.3  144.7    220.0  212.2    287.4  278.3
-//   sugar    123.2  124.2    144.2  140.7    165.8  157.4    249.4  232.0    326.3  304.2
-//   WENO3     89.0   91.1    103.4  103.1    118.3  116.1    183.9  173.2    241.0  227.0
-//   sign      99.1  100.6    114.9  113.8    131.1  127.6    199.9  186.8    261.4  243.6
+//   plain    110.4  115.0    128.1  130.1    145.8  145.3    220.4  212.4    287.9  278.3
+//   sugar    121.7  124.2    142.1  140.7    163.0  157.3    245.6  231.2    320.6  303.2
+//   WENO3     89.1   91.2    103.5  103.3    118.3  116.2    184.0  173.3    241.2  227.0
+//   sign      98.9  101.0    114.7  113.9    131.2  127.8    200.5  186.5    261.7  243.7
 constexpr long long kTileMaxNodes = 3500000;
 
 struct Tile2dSmem {
