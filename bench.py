@@ -176,7 +176,7 @@ NCU_TRAFFIC = {
     "rk_stage2": (172.9e6, _STAGE_SRC, "df81c1304f23"),
     "rk_stage3": (166.3e6, _STAGE_SRC, "df81c1304f23"),
     # 512 x 1024 adjoint workload, mean of the three stages (step records read from HBM)
-    "adj_faces": (12.65e6, ("adjoint_tile.cuh", "weno.cuh", "adjoint.cuh") + _LBM_SRC, "c9d11db0bd52"),
+    "adj_faces": (12.65e6, ("adjoint_tile.cuh", "weno.cuh", "adjoint.cuh") + _LBM_SRC, "aa0cb84a9158"),
 }
 # the 256 x 256 x 512 D3Q19 workload
 NCU_TRAFFIC_3D = {
